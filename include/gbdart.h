@@ -164,7 +164,7 @@ typedef struct {
 typedef struct {
     int32_t packet_w, packet_h;  /* pixels of one warp packet: 8x4, 4x8, 16x2, 32x1 */
     int32_t cta_warps;           /* warps per CTA: 1, 2, 4 or 8                     */
-    int32_t depth;               /* cells gathered ahead per lane: 1, 2 or 4       */
+    int32_t depth;               /* cells in flight per lane: 1, 2 or 4            */
     int32_t persistent;          /* 1 = CTAs loop over their view's tile counter;
                                     0 = one packet per warp, one launch wave    */
     int32_t regcap;              /* 1 = kernel built for at most 80 registers/thread */
@@ -185,8 +185,10 @@ typedef struct {
     int32_t group;               /* batches: time groups.  Consecutive views that
                                     differ only in observer time (same image plane,
                                     direction and grid frame; t_obs, and with it the
-                                    window, and nu_ratio free) are marched together,
-                                    up to `group` per ray: one traversal, one sum per
+                                    window, and nu_ratio free) and lie within three
+                                    snapshots of each other are marched together,
+                                    up to `group` per ray: one traversal and one
+                                    gather of the snapshots they share, one sum per
                                     view.  0 = the default, 4; 1 = every view on its
                                     own; at most 8.  A grouped view agrees with its
                                     lone render to FP32 rounding, not bitwise.       */

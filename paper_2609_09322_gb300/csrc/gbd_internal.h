@@ -11,8 +11,8 @@
 
 namespace gbd {
 
-// Largest grid edge the kernels accept; the three per-axis offset tables of a
-// volume are staged in shared memory, 4 bytes per entry.
+// Largest grid edge the kernels accept; the march tables of a volume are
+// staged in shared memory, 8 bytes per cell along each axis.
 constexpr int kMaxAxis = 4096;
 
 // A packed volume as the kernels see it.  The record of cell (ix, iy, iz) at
@@ -40,19 +40,16 @@ constexpr float kPlainGamma2 = 64.0f;
 
 // March tables.  The march steps every axis towards increasing cell index:
 // an axis the view runs down is mirrored (cell k' = n - 1 - k) on the host.
-// For each axis the tables hold the forward terms off[0 .. n-1], then two
-// sentinels, then the reversed terms off[n-1 .. 0], then two sentinels.  A
-// step onto a sentinel is a step out of the box, and the sign bit of the
-// sentinel tells the march so; the second sentinel absorbs the read-ahead
-// of the next cell's term.
-constexpr int32_t kTabSentinel = INT32_MIN;
-// Sentinels after the last staged table in shared memory (see stage_tables).
-constexpr int kTabPad = 2;
+// For each axis the tables hold, forward and then reversed, the change of the
+// layout offset at the step out of cell 0, 1, ..., n - 2 and two more entries
+// (zero): the step out of the box, and the entry a ray that has left it points
+// at.  One offset per ray then follows the march, moved by one table read per
+// step; a ray takes its first offset from axis_off.
 __host__ __device__ inline int march_table_base(const int n[3], int axis)
 {
-    return axis == 0 ? 0 : (axis == 1 ? 2 * (n[0] + 2) : 2 * (n[0] + 2) + 2 * (n[1] + 2));
+    return axis == 0 ? 0 : (axis == 1 ? 2 * (n[0] + 1) : 2 * (n[0] + 1) + 2 * (n[1] + 1));
 }
-__host__ __device__ inline int march_table_entries(const int n[3]) { return 2 * (n[0] + n[1] + n[2] + 6); }
+__host__ __device__ inline int march_table_entries(const int n[3]) { return 2 * (n[0] + n[1] + n[2] + 3); }
 
 // Bits of ViewDev::flags above the public GBD_BEAMING / GBD_LOOKBACK bits:
 // axis i is mirrored (the view's direction has s_hat_i < 0).
@@ -101,6 +98,11 @@ constexpr int kViewsPerLaunch = 128;
 // kGroupDefault when the launch does not say.
 constexpr int kGroupMax = 8;
 constexpr int kGroupDefault = 4;
+// Snapshots that a group's cell gathers and boosts once for all its members:
+// members whose observer times lie within S - 2 snapshots of each other share
+// S.  Kernels for S = 3 and S = 5; views farther apart march on their own.
+constexpr int kGroupSnapsMin = 3;
+constexpr int kGroupSnapsMax = 5;
 
 // One march launch: n_views views of one image geometry.
 struct MarchArgs {
@@ -112,11 +114,11 @@ struct MarchArgs {
     int cta_begin[kViewsPerLaunch + 1];  // first CTA of each view (or group), then the total (set by plan_march)
     int n_groups;             // 0: every view marched on its own; else time groups of consecutive views
     int group_size;           // time groups: the kernel's member limit (4 or kGroupMax)
+    int group_snaps;          // and its snapshots per cell (kGroupSnapsMin or kGroupSnapsMax)
     int group_first[kViewsPerLaunch + 1];  // group g: views group_first[g] .. group_first[g + 1] - 1
     int group_ref[kViewsPerLaunch];        // the group's reference view: the largest u_obs
     float group_win[kViewsPerLaunch][2];   // the union of the members' windows
     long long view_delta[kViewsPerLaunch]; // u_obs of the view minus that of its group's reference, Q31.32
-    int view_dhi[kViewsPerLaunch];         // view_delta >> 32 (whole epochs, rounded down)
     int persistent;           // CTAs loop over their view's tile counter
     int accumulate;           // add to out (and samples) instead of storing
     float *out;               // n_views * width * height floats

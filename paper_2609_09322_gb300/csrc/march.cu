@@ -39,6 +39,7 @@
 
 #include <algorithm>
 #include <cfloat>
+#include <type_traits>
 
 #include "gbd_internal.h"
 
@@ -87,18 +88,8 @@ struct Record;
 template <>
 struct Record<GBD_STORE_F32> {
     using T = float4;
-    static __device__ __forceinline__ T load(const void *base, long long off)
-    {
-        return __ldg(reinterpret_cast<const float4 *>(base) + off);
-    }
+    static __device__ __forceinline__ T load_at(unsigned long long a) { return __ldg(reinterpret_cast<const float4 *>(a)); }
     static __device__ __forceinline__ T zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
-    // Both snapshots of a paired block: 32 contiguous bytes.
-    static __device__ __forceinline__ void load_pair(const void *base, long long off, T &lo, T &hi)
-    {
-        const float4 *p = reinterpret_cast<const float4 *>(base) + off;
-        lo = __ldg(p);
-        hi = __ldg(p + 1);
-    }
     // D^(2 - alpha) j' with D = sqrt(1 - beta^2) / (1 + beta . s_hat) (Eq. 14).
     // 1 + beta.s_hat and 1 - beta^2 are formed with fused multiply-adds so
     // each is rounded once near its (possibly small) value.
@@ -117,33 +108,15 @@ struct Record<GBD_STORE_F32> {
     {
         return emissivity(r) * boost(r, c);
     }
-    // boosted() of two records.  Scalar: pairing the fields of two float4
-    // records for the paired float32 instructions costs register moves, and
-    // measured slower than the scalar steps.
-    static __device__ __forceinline__ float2 boosted2(const T lo, const T hi, const BoostConsts &c)
-    {
-        return make_float2(boosted(lo, c), boosted(hi, c));
-    }
 };
 
 // 8-byte record {bf16 j', f16 u_x, f16 u_y, f16 u_z}, u = Gamma beta.
 template <>
 struct Record<GBD_STORE_BF16_F16U> {
     using T = uint2;
-    static __device__ __forceinline__ T load(const void *base, long long off)
-    {
-        return __ldg(reinterpret_cast<const uint2 *>(base) + off);
-    }
     static __device__ __forceinline__ T zero() { return make_uint2(0u, 0u); }
-    // Both snapshots of a paired block: one 16-byte load (off is even).
-    static __device__ __forceinline__ void load_pair(const void *base, long long off, T &lo, T &hi)
-    {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(base) + (off >> 1));
-        lo = make_uint2(v.x, v.y);
-        hi = make_uint2(v.z, v.w);
-    }
-    // The same by byte address.
     static __device__ __forceinline__ T load_at(unsigned long long a) { return __ldg(reinterpret_cast<const uint2 *>(a)); }
+    // Both snapshots of a paired block: one 16-byte load.
     static __device__ __forceinline__ void load_pair_at(unsigned long long a, T &lo, T &hi)
     {
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(a));
@@ -268,22 +241,16 @@ __device__ __forceinline__ float fix_to_float(long long v, float inv_scale)
     return __ll2float_rn(v) * inv_scale;
 }
 
-// One term of the march tables at byte offset `cur` from `base`: shared
-// memory in the single-volume kernel, global memory when serving.
-template <bool SMEM>
+// One entry of the march tables at byte offset `cur` from `base` (shared memory).
 __device__ __forceinline__ int32_t tab_at(const int32_t *base, uint32_t cur)
 {
-    const int32_t *p = reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(base) + cur);
-    if (SMEM) return *p;
-    return __ldg(p);
+    return *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(base) + cur);
 }
 
-// Copies a volume's march tables into shared memory, followed by kTabPad
-// sentinels: the branch-free step of a lane whose ray has ended reads up to
-// two entries past the sentinel pair it stopped at.
+// Copies a volume's march tables into shared memory.
 __device__ __forceinline__ void stage_tables(int32_t *s_tab, const int32_t *src, int ntab)
 {
-    for (int i = threadIdx.x; i < ntab + kTabPad; i += blockDim.x) s_tab[i] = i < ntab ? src[i] : kTabSentinel;
+    for (int i = threadIdx.x; i < ntab; i += blockDim.x) s_tab[i] = src[i];
 }
 
 // State of one axis of a ray: the next face crossing and what changes there.
@@ -292,51 +259,14 @@ struct AxisState {
     float sn;       // s of the next crossing, relative to the anchor
     float of;       // the anchor's offset inside its cell, times the face spacing
     long long un;   // epoch coordinate at the next crossing, Q31.32
-    uint32_t cur;   // byte offset of the current cell's table term
-    int32_t o;      // table term of the current cell
-    int32_t pn;     // table term of the next cell (read ahead)
+    uint32_t cur;   // byte offset of the table entry of the step through it
 };
 
-// Steps a ray into its next cell through the face of axis 0, 1 or 2 (x0, x1,
-// else axis 2): that axis's next crossing is recomputed from its plane count
-// (never accumulated), its epoch coordinate drops by the exact per-plane
-// amount, and the table term of the cell after is read ahead.  Every update is
-// a select on the exit axis, so the lanes of a warp never diverge here;
-// recomputing an axis's crossing from an unchanged plane count reproduces it
-// (an axis the ray runs parallel to has of = -3e38 and inv_a = 0, so its
-// crossing stays at 3e38).
-template <bool SMEM>
-__device__ __forceinline__ void step_exit(AxisState (&ax)[3], bool x0, bool x1, float ia0, float ia1, float ia2,
-                                          long long du0, long long du1, long long du2, const int32_t *tab)
-{
-    const bool x2 = !x0 && !x1;
-    const uint32_t ce = x0 ? ax[0].cur : (x1 ? ax[1].cur : ax[2].cur);
-    const int32_t tn = tab_at<SMEM>(tab, ce + 8u);
-    ax[0].nkf = x0 ? ax[0].nkf + 1.0f : ax[0].nkf;
-    ax[1].nkf = x1 ? ax[1].nkf + 1.0f : ax[1].nkf;
-    ax[2].nkf = x2 ? ax[2].nkf + 1.0f : ax[2].nkf;
-    ax[0].un = x0 ? ax[0].un - du0 : ax[0].un;
-    ax[1].un = x1 ? ax[1].un - du1 : ax[1].un;
-    ax[2].un = x2 ? ax[2].un - du2 : ax[2].un;
-    ax[0].o = x0 ? ax[0].pn : ax[0].o;
-    ax[1].o = x1 ? ax[1].pn : ax[1].o;
-    ax[2].o = x2 ? ax[2].pn : ax[2].o;
-    ax[0].pn = x0 ? tn : ax[0].pn;
-    ax[1].pn = x1 ? tn : ax[1].pn;
-    ax[2].pn = x2 ? tn : ax[2].pn;
-    ax[0].cur = x0 ? ax[0].cur + 4u : ax[0].cur;
-    ax[1].cur = x1 ? ax[1].cur + 4u : ax[1].cur;
-    ax[2].cur = x2 ? ax[2].cur + 4u : ax[2].cur;
-    ax[0].sn = fmaf(ax[0].nkf, ia0, -ax[0].of);
-    ax[1].sn = fmaf(ax[1].nkf, ia1, -ax[1].of);
-    ax[2].sn = fmaf(ax[2].nkf, ia2, -ax[2].of);
-}
-
 // The box a ray is marched through, in the march frame (mirrored axes
-// mirrored), and where its table terms start: the whole grid for a direct
-// render, one region of it for the region schedule.  Along axis i the cells
-// lo[i] .. hi[i] - 1 have their terms at byte offsets cur0[i], cur0[i] + 4, ...
-// followed by two sentinels.
+// mirrored), and where its table entries start: the whole grid for a direct
+// render, one region of it for the region schedule.  Along axis i the steps out
+// of cells lo[i] .. hi[i] - 1 have their entries at byte offsets cur0[i],
+// cur0[i] + 4, ..., and one more entry follows (of any value).
 struct RayBox {
     int lo[3], hi[3];
     uint32_t cur0[3];
@@ -351,17 +281,20 @@ __device__ __forceinline__ RayBox grid_box(const VolDev &vol, const ViewDev &V)
         const bool mirrored = (V.flags & (kFlagMirror0 << i)) != 0u;
         B.lo[i] = 0;
         B.hi[i] = vol.n[i];
-        B.cur0[i] = 4u * static_cast<uint32_t>(march_table_base(vol.n, i) + (mirrored ? vol.n[i] + 2 : 0));
+        B.cur0[i] = 4u * static_cast<uint32_t>(march_table_base(vol.n, i) + (mirrored ? vol.n[i] + 1 : 0));
     }
     return B;
 }
 
-// State of a ray during the march: per axis the next crossing, the current
-// cell's chord start (the latest face crossed) and its epoch coordinate.
+// State of a ray during the march: per axis the next crossing, the layout
+// offset of the current cell, its chord start (the latest face crossed) and
+// the epoch coordinate there.
 struct RayState {
     AxisState ax[3];
+    uint32_t sum;      // layout offset of the current cell (the sum of its three axis terms)
     float s_cur;       // s of the latest face crossed
-    long long u_cur;   // epoch coordinate there, Q31.32
+    float s_end;       // s of the box face through which the ray leaves
+    long long u_cur;   // epoch coordinate at s_cur, Q31.32
     long long u_a;     // epoch coordinate at the anchor (s = 0), Q31.32
     bool alive;
 #ifdef GBD_CHECKED
@@ -369,12 +302,83 @@ struct RayState {
 #endif
 };
 
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float r;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+// The face through which a ray leaves its cell: the nearest of the three next
+// crossings, ties to the lowest axis (the zero-length chord that follows adds
+// nothing).  No axis is set for a lane whose ray has ended.
+struct ExitFace {
+    bool x0, x1, x2;
+    float s;
+};
+__device__ __forceinline__ ExitFace exit_face(const AxisState (&ax)[3], bool alive)
+{
+    ExitFace X;
+    X.s = min3(ax[0].sn, ax[1].sn, ax[2].sn);
+    X.x0 = alive & (ax[0].sn <= X.s);
+    X.x1 = alive & !X.x0 & (ax[1].sn <= X.s);
+    X.x2 = alive & !X.x0 & !X.x1;
+    return X;
+}
+
+// Steps a ray into its next cell through face X: the exit axis's next crossing
+// is recomputed from its plane count (never accumulated), and the table entry
+// of the step moves the cell's layout offset.  Every update is a select on the
+// exit axis, so the lanes of a warp never diverge here; recomputing an axis's
+// crossing from an unchanged plane count reproduces it (an axis the ray runs
+// parallel to has of = -3e38 and inv_a = 0, so its crossing stays at 3e38).
+// A lane whose ray has ended keeps its crossings and cursors and reads the
+// table at the cursor it stopped at; its layout offset is never used again.
+__device__ __forceinline__ void step_lite(RayState &R, const ExitFace &X, float ia0, float ia1, float ia2,
+                                          const int32_t *tab)
+{
+    AxisState (&ax)[3] = R.ax;
+    const uint32_t ce = X.x0 ? ax[0].cur : (X.x1 ? ax[1].cur : ax[2].cur);
+    R.sum += static_cast<uint32_t>(tab_at(tab, ce));
+    ax[0].nkf = X.x0 ? ax[0].nkf + 1.0f : ax[0].nkf;
+    ax[1].nkf = X.x1 ? ax[1].nkf + 1.0f : ax[1].nkf;
+    ax[2].nkf = X.x2 ? ax[2].nkf + 1.0f : ax[2].nkf;
+    ax[0].cur = X.x0 ? ax[0].cur + 4u : ax[0].cur;
+    ax[1].cur = X.x1 ? ax[1].cur + 4u : ax[1].cur;
+    ax[2].cur = X.x2 ? ax[2].cur + 4u : ax[2].cur;
+    ax[0].sn = fmaf(ax[0].nkf, ia0, -ax[0].of);
+    ax[1].sn = fmaf(ax[1].nkf, ia1, -ax[1].of);
+    ax[2].sn = fmaf(ax[2].nkf, ia2, -ax[2].of);
+#ifdef GBD_CHECKED
+    R.kc[0] += X.x0 ? R.kd[0] : 0;
+    R.kc[1] += X.x1 ? R.kd[1] : 0;
+    R.kc[2] += X.x2 ? R.kd[2] : 0;
+#endif
+}
+
+// step_lite with the exact epoch coordinate of each axis: it drops by the
+// exact per-plane amount.
+__device__ __forceinline__ void step_exact(RayState &R, const ExitFace &X, float ia0, float ia1, float ia2,
+                                           long long du0, long long du1, long long du2, const int32_t *tab)
+{
+    step_lite(R, X, ia0, ia1, ia2, tab);
+    R.ax[0].un = X.x0 ? R.ax[0].un - du0 : R.ax[0].un;
+    R.ax[1].un = X.x1 ? R.ax[1].un - du1 : R.ax[1].un;
+    R.ax[2].un = X.x2 ? R.ax[2].un - du2 : R.ax[2].un;
+}
+
 // Ray set-up, once per ray, no float64: the anchor at the later of the box
 // entry and the window start [win_lo, win_hi] (a view's own window, or the
 // union of a group's), its cell and crossings, and the leading empty chords
 // stepped through, so that the march proper starts on the first cell whose
 // chord is positive.
-template <bool SMEM>
+//
+// s_end is where the ray leaves the box: along axis i the crossing of the box's
+// upper face is the crossing of plane hi[i] - k, computed from that plane count
+// exactly as the march will, and the nearest of the three is s_end.  A
+// crossing before s_end is therefore not the last one of its axis, and a ray
+// that stops at the first crossing at or past s_end never steps a cursor past
+// the entry behind its box's last cell: one float comparison per step keeps
+// every gather inside the box.
 __device__ __forceinline__ void setup_ray(RayState &R, const VolDev &vol, const ViewDev &V, const RayBox &B, int p,
                                           int q, bool in_image, float win_lo, float win_hi,
                                           const int32_t *__restrict__ tab)
@@ -383,9 +387,6 @@ __device__ __forceinline__ void setup_ray(RayState &R, const VolDev &vol, const 
     bool &alive = R.alive;
     float &s_cur = R.s_cur;
     long long &u_cur = R.u_cur;
-#ifdef GBD_CHECKED
-    int (&kc)[3] = R.kc;
-#endif
     alive = in_image;
     // Pixel position on the image plane in grid-index units (Q24.40, exact
     // integer arithmetic from the per-view constants), in the frame where
@@ -422,19 +423,27 @@ __device__ __forceinline__ void setup_ray(RayState &R, const VolDev &vol, const 
     R.u_a = u_a;
     s_cur = -3.0e38f;  // the latest entry face of the anchor cell
     u_cur = 0;
+    R.sum = 0;
+    R.s_end = 3.0e38f;
+    const int32_t *off = vol.axis_off;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const bool moving = V.inv_a[i] != 0.f;
+        const bool mirrored = (V.flags & (kFlagMirror0 << i)) != 0u;
         const long long ga = moving ? g0[i] + dd_mul_fix(sa, V.a_hi[i], V.a_lo[i], kTwo40) : g0[i];
         int k = static_cast<int>(ga >> 40);
         k = min(max(k, B.lo[i]), B.hi[i] - 1);
         const float o = fix_to_float(ga - (static_cast<long long>(k) << 40), kInv2p40);
         AxisState &A = ax[i];
         A.nkf = 1.0f;
-        A.of = o * V.inv_a[i];
+        // Rounded products and differences, never contracted: this first
+        // crossing, the recomputed ones and s_end have to be one function of
+        // the plane count, or a ray could pass its last face unseen.
+        A.of = __fmul_rn(o, V.inv_a[i]);
         if (moving) {
-            A.sn = V.inv_a[i] - A.of;
+            A.sn = __fsub_rn(V.inv_a[i], A.of);
             A.un = u_a - dd_mul_fix(1.0f - o, V.w_hi[i], V.w_lo[i], kTwo32);
+            R.s_end = fminf(R.s_end, fmaf(static_cast<float>(B.hi[i] - k), V.inv_a[i], -A.of));
             // the anchor cell's entry face along this axis (plane nk = 0)
             if (-A.of > s_cur) {
                 s_cur = -A.of;
@@ -442,67 +451,71 @@ __device__ __forceinline__ void setup_ray(RayState &R, const VolDev &vol, const 
             }
         } else {
             A.of = -3.0e38f;     // with inv_a = 0: the crossing stays at 3e38,
-            A.sn = 3.0e38f;      // never the nearest face ...
-            A.un = LLONG_MIN / 2;  // ... and ends the ray if it ever were
+            A.sn = 3.0e38f;      // never the nearest face
+            A.un = LLONG_MIN / 2;
         }
         A.cur = B.cur0[i] + 4u * static_cast<uint32_t>(k - B.lo[i]);
-        A.o = 0;
-        A.pn = 0;
-        if (alive) {
-            A.o = tab_at<SMEM>(tab, A.cur);
-            A.pn = tab_at<SMEM>(tab, A.cur + 4u);
-        }
+        R.sum += static_cast<uint32_t>(__ldg(off + (mirrored ? vol.n[i] - 1 - k : k)));
+        off += vol.n[i];
 #ifdef GBD_CHECKED
-        kc[i] = (V.flags & (kFlagMirror0 << i)) ? vol.n[i] - 1 - k : k;
+        R.kc[i] = mirrored ? vol.n[i] - 1 - k : k;
+        R.kd[i] = mirrored ? -1 : 1;
 #endif
     }
-    const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
-    const long long du0 = V.du[0], du1 = V.du[1], du2 = V.du[2];
-#ifdef GBD_CHECKED
-    const int kd0 = (V.flags & kFlagMirror0) ? -1 : 1;
-    const int kd1 = (V.flags & (kFlagMirror0 << 1)) ? -1 : 1;
-    const int kd2 = (V.flags & (kFlagMirror0 << 2)) ? -1 : 1;
-    R.kd[0] = kd0;
-    R.kd[1] = kd1;
-    R.kd[2] = kd2;
-#endif
 
     // Leading empty chords: when the anchor cell was clamped onto the grid, or
     // the anchor sits on a face, the ray can leave a cell along one axis before
     // it has entered it along another.  Those cells are stepped through until
     // the nearest exit lies past the latest entry; from there on the exits
     // only increase, so every chord of the march proper starts at the end of
-    // the one before.  Each step moves one table cursor up, and a sentinel
-    // stops the ray at the box face, so the loop is bounded by the grid.
+    // the one before.  Each step moves one table cursor up, and s_end stops
+    // the ray at the box face, so the loop is bounded by the grid.
     if (alive) {
         for (int guard = B.hi[0] + B.hi[1] + B.hi[2] + 4; guard > 0; --guard) {
-            const bool x0 = ax[0].sn <= ax[1].sn && ax[0].sn <= ax[2].sn;
-            const bool x1 = !x0 && ax[1].sn <= ax[2].sn;
-            const float s_exit = x0 ? ax[0].sn : (x1 ? ax[1].sn : ax[2].sn);
-            if (s_exit > s_cur) break;
-            step_exit<SMEM>(ax, x0, x1, ia0, ia1, ia2, du0, du1, du2, tab);
-#ifdef GBD_CHECKED
-            kc[0] += x0 ? kd0 : 0;
-            kc[1] += x1 ? kd1 : 0;
-            kc[2] += (!x0 && !x1) ? kd2 : 0;
-#endif
-            if ((ax[0].o | ax[1].o | ax[2].o) < 0) {
+            const ExitFace X = exit_face(ax, true);
+            if (X.s > s_cur) break;
+            if (X.s >= R.s_end) {
                 alive = false;
                 break;
             }
+            step_exact(R, X, V.inv_a[0], V.inv_a[1], V.inv_a[2], V.du[0], V.du[1], V.du[2], tab);
         }
     }
 }
 
+// Where the march of a ray may stop: at s_end, or past the last time that
+// reaches a snapshot (u < -1).  Beyond that time no chord has a weight, so the
+// bound only has to lie at or past it: it is taken a few float roundings late.
+__device__ __forceinline__ float march_end(const RayState &R, float kk)
+{
+    const float c0 = fix_to_float(R.u_a, 1.0f / kTwo32);
+    const float s_stop = kk > 0.f ? (c0 + 1.0f + 1e-6f * (fabsf(c0) + 1.0f)) / kk : 3.0e38f;
+    return fminf(R.s_end, s_stop);
+}
+
+// Byte address of the unit of UNIT bytes (a record, or a pair of them) at layout
+// offset `sum` of block `blk`, blocks blk_bytes apart.  The block term is one 64-bit
+// product of bytes: the same address as (blk * units + sum) << log2(UNIT), in
+// units of a shifted stride, was miscompiled in some kernels (CUDA 13.0: the
+// shift applied to the stride and again to the product).
+template <unsigned UNIT>
+__device__ __forceinline__ unsigned long long rec_addr(unsigned long long base, int blk, long long blk_bytes,
+                                                       uint32_t sum)
+{
+    return base + static_cast<unsigned long long>(static_cast<long long>(blk) * blk_bytes) +
+           static_cast<unsigned long long>(sum) * UNIT;
+}
+
 // The float epoch coordinate of the bfloat16/float16 march: u(s) = c0 -
 // kk s along the ray (s from the anchor), so that the chord midpoint's is
-// c0 + mkk (s_cur + s_exit) with mkk = -kk / 2; the ray has passed the last
-// time that reaches a snapshot (u < -1) beyond s_stop.  c0 is the exact
+// c0 + mkk (s_cur + s_exit) with mkk = -kk / 2; the ray stops at the first
+// crossing at or past s_lim, the nearer of the box face and the first float
+// past s_stop = (c0 + 1) / kk, the last time that reaches a snapshot (u = -1).  c0 is the exact
 // coordinate at the anchor rounded to float: the coordinate is off by at most
 // a few float ulps of M (2e-6 snapshots at M = 16), against the 2^-9 and
 // 2^-11 resolution of the stored j' and u.
 struct EpochLine {
-    float c0, mkk, s_stop;
+    float c0, mkk, s_lim;
 };
 __device__ __forceinline__ EpochLine epoch_line(const RayState &R, const ViewDev &V)
 {
@@ -510,36 +523,58 @@ __device__ __forceinline__ EpochLine epoch_line(const RayState &R, const ViewDev
     const float kk = V.kk_hi;
     L.c0 = fix_to_float(R.u_a, 1.0f / kTwo32);
     L.mkk = -0.5f * kk;
-    L.s_stop = kk > 0.f ? (L.c0 + 1.0f) / kk : 3.0e38f;
+    L.s_lim = R.s_end;
+    if (kk > 0.f) {
+        const float s_stop = (L.c0 + 1.0f) / kk;
+        // the next float up: s <= s_stop is s < next
+        const int b = __float_as_int(s_stop);
+        const float next = s_stop > 0.f ? __int_as_float(b + 1) : (s_stop < 0.f ? __int_as_float(b - 1) : FLT_MIN);
+        L.s_lim = fminf(L.s_lim, next);
+    }
     return L;
 }
 
-// One step of the bfloat16/float16 march through the face of axis 0, 1 or 2
-// (x0, x1, x2, at most one of them set; none once the ray has ended): the
-// plane count and crossing of that axis, and its table terms.  Every lane
-// executes it; a lane that takes no step changes nothing, and its read of
-// the table stays within the padding after the last sentinel.
-template <bool SMEM>
-__device__ __forceinline__ void step_lite(AxisState (&ax)[3], bool x0, bool x1, bool x2, float ia0, float ia1,
-                                          float ia2, const int32_t *tab)
+// floor(u) + 1 as an integer, and the fraction w = u - floor(u), on the FMA pipe:
+// u + 1.5 * 2^23 rounded down holds floor(u) in its low mantissa bits for
+// |u| < 2^22 (snapshot counts end at 10^6); for any other u the integer lies outside
+// [0, 10^6], so a range test on it still fails.
+__device__ __forceinline__ int floor_plus1(float u, float &w)
 {
-    const uint32_t ce = x0 ? ax[0].cur : (x1 ? ax[1].cur : ax[2].cur);
-    const int32_t tn = tab_at<SMEM>(tab, ce + 8u);
-    ax[0].nkf = x0 ? ax[0].nkf + 1.0f : ax[0].nkf;
-    ax[1].nkf = x1 ? ax[1].nkf + 1.0f : ax[1].nkf;
-    ax[2].nkf = x2 ? ax[2].nkf + 1.0f : ax[2].nkf;
-    ax[0].o = x0 ? ax[0].pn : ax[0].o;
-    ax[1].o = x1 ? ax[1].pn : ax[1].o;
-    ax[2].o = x2 ? ax[2].pn : ax[2].o;
-    ax[0].pn = x0 ? tn : ax[0].pn;
-    ax[1].pn = x1 ? tn : ax[1].pn;
-    ax[2].pn = x2 ? tn : ax[2].pn;
-    ax[0].cur = x0 ? ax[0].cur + 4u : ax[0].cur;
-    ax[1].cur = x1 ? ax[1].cur + 4u : ax[1].cur;
-    ax[2].cur = x2 ? ax[2].cur + 4u : ax[2].cur;
-    ax[0].sn = fmaf(ax[0].nkf, ia0, -ax[0].of);
-    ax[1].sn = fmaf(ax[1].nkf, ia1, -ax[1].of);
-    ax[2].sn = fmaf(ax[2].nkf, ia2, -ax[2].of);
+    const float t = __fadd_rd(u, 12582912.0f);
+    w = u - (t - 12582912.0f);
+    return static_cast<int>(static_cast<unsigned>(__float_as_int(t)) - 0x4B3FFFFFu);
+}
+
+// The march's loop.  A stage is H cells of every lane: gather() traverses them
+// and issues the loads of their records, evaluate() boosts and sums them.  PIPED: two
+// stages alternate, and each is evaluated after the next one has been gathered, so that
+// its loads have the evaluation of the stage before and the traversal of
+// the stage after to arrive in.  What bounds the march is waiting for its gathers (issue
+// slots half used); a lane has as many cells in flight as one that gathers 2 H
+// and then evaluates 2 H, but does not stand still for them (one 1024^2 image of 512^3 x 8
+// bfloat16/float16 records: 865 us with 4 cells gathered and evaluated, 809 as 2 + 2; region schedule
+// of 256 float32 views: 20.1 -> 19.4 ms).
+template <bool PIPED, class Stage, class Gather, class Evaluate>
+__device__ __forceinline__ void run_stages(const bool &alive, Gather gather, Evaluate evaluate)
+{
+    Stage a;
+    if constexpr (PIPED) {
+        if (!__any_sync(kFull, alive)) return;
+        Stage b;
+        gather(a);
+        while (__any_sync(kFull, alive)) {
+            gather(b);
+            evaluate(a);
+            gather(a);
+            evaluate(b);
+        }
+        evaluate(a);
+    } else {
+        while (__any_sync(kFull, alive)) {
+            gather(a);
+            evaluate(a);
+        }
+    }
 }
 
 // The march of march_ray for bfloat16/float16 records (see the file
@@ -554,17 +589,12 @@ __device__ __forceinline__ void march_ray_bf16(const VolDev &vol, const ViewDev 
     using Rec = Record<GBD_STORE_BF16_F16U>;
     const bool in_image = (p < width) && (q < height);
     RayState R;
-    setup_ray<true>(R, vol, V, B, p, q, in_image, V.win_lo, V.win_hi, tab);
-    AxisState (&ax)[3] = R.ax;
+    setup_ray(R, vol, V, B, p, q, in_image, V.win_lo, V.win_hi, tab);
     bool alive = R.alive;
     float s_cur = R.s_cur;
     const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
     const EpochLine L = epoch_line(R, V);
     const int M = vol.M;
-#ifdef GBD_CHECKED
-    int (&kc)[3] = R.kc;
-    const int kd0 = R.kd[0], kd1 = R.kd[1], kd2 = R.kd[2];
-#endif
 
     BoostConsts bc;
     bc.shx = V.sh_hi[0]; bc.shy = V.sh_hi[1]; bc.shz = V.sh_hi[2];
@@ -573,214 +603,71 @@ __device__ __forceinline__ void march_ray_bf16(const VolDev &vol, const ViewDev 
     bc.beaming = (V.flags & GBD_BEAMING) != 0u;
     bc.plain = PLAIN;
 
-    // block b starts at byte recb + b es_bytes; a cell's record (paired: its
-    // record pair) is kUnit bytes at its layout offset
-    constexpr unsigned long long kUnit = PAIRED ? 16ull : 8ull;
-    const unsigned long long recb = reinterpret_cast<unsigned long long>(vol.rec);
-    const long long es_bytes = vol.epoch_stride * 8LL;
+    // Block b of the record array (paired: of record pairs) starts b es_bytes
+    // from the base.  A sample's lower snapshot m_bar is bp - 1: unpaired, it
+    // lies in block bp - 1 and the upper one in block bp; paired, both lie in
+    // block bp.
+    constexpr unsigned kUnit = PAIRED ? 16 : 8;
+    const long long es_bytes = vol.epoch_stride * 8;
+    const unsigned long long base = reinterpret_cast<unsigned long long>(vol.rec) - (PAIRED ? 0 : es_bytes);
 
     float acc = 0.f;
     uint32_t count = 0;
-    while (__any_sync(kFull, alive)) {
-        unsigned long long pa[DEPTH];
-        float wgt[DEPTH], dsv[DEPTH];
-        bool has_lo[DEPTH], has_hi[DEPTH];
+    constexpr int H = DEPTH > 1 ? DEPTH / 2 : 1;  // cells per stage (see run_stages)
+    struct Stage {
+        float wgt[H], dsv[H];
+        bool has[H];
+        typename Rec::T rlo[H], rhi[H];
+    };
+    auto gather = [&](Stage &T) {
 #pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            // the nearest face (ties to the lowest axis), the chord, and the
-            // epoch coordinate at the chord midpoint: m_bar + w
-            const bool x0 = alive && ax[0].sn <= ax[1].sn && ax[0].sn <= ax[2].sn;
-            const bool x1 = alive && !x0 && ax[1].sn <= ax[2].sn;
-            const bool x2 = alive && !x0 && !x1;
-            const float s_exit = x0 ? ax[0].sn : (x1 ? ax[1].sn : ax[2].sn);
-            const float ds = s_exit - s_cur;
-            const float um = fmaf(L.mkk, s_cur + s_exit, L.c0);
-            const float fl = floorf(um);
-            const float w = um - fl;
-            const int mb = static_cast<int>(fl);
+        for (int d = 0; d < H; ++d) {
+            // the nearest face, the chord, and the epoch coordinate at the
+            // chord midpoint: m_bar + w
+            const ExitFace X = exit_face(R.ax, alive);
+            const float ds = X.s - s_cur;
+            const float um = fmaf(L.mkk, s_cur + X.s, L.c0);
+            float w;
+            const int bp = floor_plus1(um, w);
             // -1 <= m_bar <= M - 1; snapshots m_bar (weight 1 - w) and m_bar + 1 (w)
-            const bool take = alive && ds > 0.f && static_cast<unsigned>(mb + 1) <= static_cast<unsigned>(M);
-            has_lo[d] = take && mb >= 0;
-            has_hi[d] = take && mb < M - 1 && w != 0.f;
+            const bool take = alive & (ds > 0.f) & (static_cast<unsigned>(bp) <= static_cast<unsigned>(M));
+            bool has_lo = take & (bp != 0);
+            bool has_hi = take & (bp < M) & (w != 0.f);
 #ifdef GBD_CHECKED
-            if ((has_lo[d] && !check_cell(vol, err_word, kc[0], kc[1], kc[2], mb)) ||
-                (has_hi[d] && !check_cell(vol, err_word, kc[0], kc[1], kc[2], mb + 1)))
-                has_lo[d] = has_hi[d] = false;
-            kc[0] += x0 ? kd0 : 0;
-            kc[1] += x1 ? kd1 : 0;
-            kc[2] += x2 ? kd2 : 0;
+            if ((has_lo && !check_cell(vol, err_word, R.kc[0], R.kc[1], R.kc[2], bp - 1)) ||
+                (has_hi && !check_cell(vol, err_word, R.kc[0], R.kc[1], R.kc[2], bp)))
+                has_lo = has_hi = false;
 #endif
-            const int sum = ax[0].o + ax[1].o + ax[2].o;
-            // unpaired: snapshot m at block m; paired: snapshots mb and mb + 1
-            // side by side in block mb + 1
-            pa[d] = recb + static_cast<unsigned long long>(static_cast<long long>(PAIRED ? mb + 1 : mb) * es_bytes) +
-                    static_cast<unsigned long long>(static_cast<uint32_t>(sum)) * kUnit;
-            wgt[d] = take ? w : 0.f;
-            dsv[d] = take ? ds : 0.f;
-            step_lite<true>(ax, x0, x1, x2, ia0, ia1, ia2, tab);
-            s_cur = s_exit;
-            // past the last time that reaches a snapshot, or out of the box
-            alive = alive && s_exit <= L.s_stop && (ax[0].o | ax[1].o | ax[2].o) >= 0;
-        }
-        typename Rec::T rlo[DEPTH], rhi[DEPTH];
-#pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            rlo[d] = Rec::zero();
-            rhi[d] = Rec::zero();
+            const unsigned long long pa = rec_addr<kUnit>(base, bp, es_bytes, R.sum);
+            T.wgt[d] = take ? w : 0.f;
+            T.dsv[d] = take ? ds : 0.f;
+            T.has[d] = has_lo | has_hi;
+            T.rlo[d] = Rec::zero();
+            T.rhi[d] = Rec::zero();
             if (PAIRED) {
-                if (has_lo[d] || has_hi[d]) Rec::load_pair_at(pa[d], rlo[d], rhi[d]);
+                if (has_lo | has_hi) Rec::load_pair_at(pa, T.rlo[d], T.rhi[d]);
             } else {
-                if (has_lo[d]) rlo[d] = Rec::load_at(pa[d]);
-                if (has_hi[d]) rhi[d] = Rec::load_at(pa[d] + es_bytes);
+                if (has_lo) T.rlo[d] = Rec::load_at(pa);
+                if (has_hi) T.rhi[d] = Rec::load_at(pa + es_bytes);
             }
+            step_lite(R, X, ia0, ia1, ia2, tab);
+            s_cur = X.s;
+            alive = alive & (X.s < L.s_lim);
         }
-        // A snapshot a sample does not read is a zero record (boosted value
-        // exactly 0), and a sample not taken has weight and chord 0.
+    };
+    // A snapshot a sample does not read is a zero record (boosted value
+    // exactly 0), and a sample not taken has weight and chord 0.
+    auto evaluate = [&](const Stage &T) {
 #pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            const float2 vv = PLAIN ? Rec::boosted2_plain(rlo[d], rhi[d], bc) : Rec::boosted2(rlo[d], rhi[d], bc);
-            const float v = fmaf(wgt[d], vv.y - vv.x, vv.x);  // Eq. 8
-            acc = fmaf(v, dsv[d], acc);
-            count += (has_lo[d] || has_hi[d]) ? 1u : 0u;
+        for (int d = 0; d < H; ++d) {
+            const float2 vv = PLAIN ? Rec::boosted2_plain(T.rlo[d], T.rhi[d], bc) : Rec::boosted2(T.rlo[d], T.rhi[d], bc);
+            const float v = fmaf(T.wgt[d], vv.y - vv.x, vv.x);  // Eq. 8
+            acc = fmaf(v, T.dsv[d], acc);
+            count += T.has[d] ? 1u : 0u;
         }
-    }
+    };
+    run_stages<(DEPTH > 1), Stage>(alive, gather, evaluate);
 
-    if (in_image) {
-        const long long pix = static_cast<long long>(q) * width + p;
-        if (PARTIAL) {
-            if (count > 0u) atomicAdd(out_img + pix, acc);
-        } else if (accumulate) {
-            out_img[pix] += V.prefactor * acc;
-            if (cnt_img) cnt_img[pix] += count;
-        } else {
-            out_img[pix] = V.prefactor * acc;
-            if (cnt_img) cnt_img[pix] = count;
-        }
-    }
-}
-
-// step_lite with the exact epoch coordinate of each axis (float32 march).
-template <bool SMEM>
-__device__ __forceinline__ void step_nb(AxisState (&ax)[3], bool x0, bool x1, bool x2, float ia0, float ia1,
-                                        float ia2, long long du0, long long du1, long long du2, const int32_t *tab)
-{
-    step_lite<SMEM>(ax, x0, x1, x2, ia0, ia1, ia2, tab);
-    ax[0].un = x0 ? ax[0].un - du0 : ax[0].un;
-    ax[1].un = x1 ? ax[1].un - du1 : ax[1].un;
-    ax[2].un = x2 ? ax[2].un - du2 : ax[2].un;
-}
-
-// The march of march_ray for float32 records without branches: the step of
-// march_ray_bf16 (every lane executes it; a lane whose ray has ended takes no
-// step and reads no record) with the exact Q31.32 epoch coordinate, the
-// float32 Doppler factor of Eq. 14 and the compensated sum.  Its arithmetic
-// is that of the branching form, value for value.
-template <int DEPTH, bool PAIRED, bool PARTIAL>
-__device__ __forceinline__ void march_ray_f32(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
-                                              int width, int height, float *out_img, uint32_t *cnt_img,
-                                              int *err_word, const int32_t *__restrict__ tab, bool accumulate)
-{
-    using Rec = Record<GBD_STORE_F32>;
-    const bool in_image = (p < width) && (q < height);
-    RayState R;
-    setup_ray<true>(R, vol, V, B, p, q, in_image, V.win_lo, V.win_hi, tab);
-    AxisState (&ax)[3] = R.ax;
-    bool alive = R.alive;
-    float s_cur = R.s_cur;
-    long long u_cur = R.u_cur;
-    const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
-    const long long du0 = V.du[0], du1 = V.du[1], du2 = V.du[2];
-    const int Mm1 = vol.M - 1;
-#ifdef GBD_CHECKED
-    int (&kc)[3] = R.kc;
-    const int kd0 = R.kd[0], kd1 = R.kd[1], kd2 = R.kd[2];
-#endif
-    BoostConsts bc;
-    bc.shx = V.sh_hi[0]; bc.shy = V.sh_hi[1]; bc.shz = V.sh_hi[2];
-    bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
-    bc.expo = V.expo;
-    bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-    bc.plain = false;
-    // block b starts at byte recb + b es_bytes; a cell's record (paired: its
-    // record pair) is kUnit bytes at its layout offset.  Paired: a sample that
-    // reads no snapshot loads the zero record pair after the last block
-    // (faster for 32-byte pairs than a predicated load).
-    constexpr unsigned long long kUnit = PAIRED ? 32ull : 16ull;
-    const unsigned long long recb = reinterpret_cast<unsigned long long>(vol.rec);
-    const long long es_bytes = vol.epoch_stride * 16LL;
-    const unsigned long long zero_addr = recb + static_cast<unsigned long long>((vol.M + 1) * es_bytes);
-
-    float acc = 0.f, comp = 0.f;
-    uint32_t count = 0;
-    while (__any_sync(kFull, alive)) {
-        unsigned long long pa[DEPTH];
-        float wgt[DEPTH], dsv[DEPTH];
-        bool has_lo[DEPTH], has_hi[DEPTH];
-#pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            const bool x0 = alive && ax[0].sn <= ax[1].sn && ax[0].sn <= ax[2].sn;
-            const bool x1 = alive && !x0 && ax[1].sn <= ax[2].sn;
-            const bool x2 = alive && !x0 && !x1;
-            const float s_exit = x0 ? ax[0].sn : (x1 ? ax[1].sn : ax[2].sn);
-            const long long u_exit = x0 ? ax[0].un : (x1 ? ax[1].un : ax[2].un);
-            const float ds = s_exit - s_cur;
-            // epoch coordinate at the chord midpoint: m_bar + w, w in [0, 1)
-            const long long um = (u_cur + u_exit) >> 1;
-            const int mb = static_cast<int>(um >> 32);
-            const uint32_t frac = static_cast<uint32_t>(um);
-            const float w = static_cast<float>(frac) * 2.3283064365386963e-10f;
-            // -1 <= m_bar <= M - 1 (at u = -1 exactly both weights vanish)
-            const bool take = alive && ds > 0.f && static_cast<unsigned>(mb + 1) <= static_cast<unsigned>(Mm1 + 1);
-            has_lo[d] = take && mb >= 0;
-            has_hi[d] = take && mb < Mm1 && frac != 0u;
-#ifdef GBD_CHECKED
-            if ((has_lo[d] && !check_cell(vol, err_word, kc[0], kc[1], kc[2], mb)) ||
-                (has_hi[d] && !check_cell(vol, err_word, kc[0], kc[1], kc[2], mb + 1)))
-                has_lo[d] = has_hi[d] = false;
-            kc[0] += x0 ? kd0 : 0;
-            kc[1] += x1 ? kd1 : 0;
-            kc[2] += x2 ? kd2 : 0;
-#endif
-            const int sum = ax[0].o + ax[1].o + ax[2].o;
-            const unsigned long long a = recb + static_cast<unsigned long long>(static_cast<long long>(PAIRED ? mb + 1 : mb) * es_bytes) +
-                    static_cast<unsigned long long>(static_cast<uint32_t>(sum)) * kUnit;
-            pa[d] = PAIRED ? ((has_lo[d] || has_hi[d]) ? a : zero_addr) : a;
-            wgt[d] = w;
-            dsv[d] = ds;
-            step_nb<true>(ax, x0, x1, x2, ia0, ia1, ia2, du0, du1, du2, tab);
-            s_cur = s_exit;
-            u_cur = u_exit;
-            // past the last time that reaches a snapshot (u < -1), or out of the box
-            alive = alive && static_cast<int>(u_exit >> 32) >= -1 && (ax[0].o | ax[1].o | ax[2].o) >= 0;
-        }
-        typename Rec::T rlo[DEPTH], rhi[DEPTH];
-#pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            if (PAIRED) {
-                const float4 *ptr = reinterpret_cast<const float4 *>(pa[d]);
-                rlo[d] = __ldg(ptr);
-                rhi[d] = __ldg(ptr + 1);
-            } else {
-                rlo[d] = has_lo[d] ? __ldg(reinterpret_cast<const float4 *>(pa[d])) : Rec::zero();
-                rhi[d] = has_hi[d] ? __ldg(reinterpret_cast<const float4 *>(pa[d] + es_bytes)) : Rec::zero();
-            }
-        }
-#pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            // a snapshot the sample does not read is a zero record (boosted
-            // value exactly 0); the compensated sum takes the sample only where
-            // it read one
-            const float vlo = Rec::boosted(rlo[d], bc);
-            const float vhi = Rec::boosted(rhi[d], bc);
-            const float v = fmaf(wgt[d], vhi - vlo, vlo);  // Eq. 8
-            const float y = fmaf(v, dsv[d], -comp);
-            const float t = acc + y;
-            const bool take = has_lo[d] || has_hi[d];
-            comp = take ? (t - acc) - y : comp;
-            acc = take ? t : acc;
-            count += take ? 1u : 0u;
-        }
-    }
     if (in_image) {
         const long long pix = static_cast<long long>(q) * width + p;
         if (PARTIAL) {
@@ -802,7 +689,7 @@ __device__ __forceinline__ void march_ray_f32(const VolDev &vol, const ViewDev &
 // successive launches land in launch order).  PARTIAL: adds the ray's sum over
 // the box, without the prefactor, to out_img[pixel] if the ray sampled at
 // least one cell there (one region per slot and ray, so the add lands on
-// zero).  tab points at the march tables (shared memory when SMEM).
+// zero).  tab points at the march tables in shared memory.
 //
 // NCH > 0 (vector renders, Sec. 2.1): the volume carries NCH more emissivity
 // channels sharing its velocity; each is summed with the same weights and
@@ -818,215 +705,148 @@ struct ChanPtrs {
     uint32_t *touch;
 };
 
-template <int STORE, int DEPTH, bool PAIRED, bool SMEM, bool PARTIAL = false, int NCH = 0, bool TOUCH = false>
-__device__ __forceinline__ void march_ray(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
-                                          int width, int height, float *out_img, uint32_t *cnt_img, int *err_word,
-                                          const int32_t *__restrict__ tab, bool accumulate = false,
-                                          const ChanPtrs ch = ChanPtrs{nullptr, 0, 0, nullptr})
+// The march without branches (every lane executes each step; a lane whose ray
+// has ended takes no step and reads no record), with the exact Q31.32 epoch
+// coordinate, the records' own Doppler factor and compensated sums: float32
+// records, and the vector and memory-analysis forms of both stores.
+template <int STORE, int DEPTH, bool PAIRED, bool PARTIAL, int NCH, bool TOUCH>
+__device__ __forceinline__ void march_ray_exact(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
+                                                int width, int height, float *out_img, uint32_t *cnt_img,
+                                                int *err_word, const int32_t *__restrict__ tab, bool accumulate,
+                                                const ChanPtrs ch)
 {
-    if constexpr (STORE == GBD_STORE_BF16_F16U && NCH == 0 && !TOUCH && SMEM) {
-        if (vol.plain_boost)
-            march_ray_bf16<DEPTH, PAIRED, PARTIAL, true>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
-                                                         tab, accumulate);
-        else
-            march_ray_bf16<DEPTH, PAIRED, PARTIAL, false>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
-                                                          tab, accumulate);
-        return;
-    }
-    if constexpr (STORE == GBD_STORE_F32 && NCH == 0 && !TOUCH && SMEM) {
-        march_ray_f32<DEPTH, PAIRED, PARTIAL>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word, tab,
-                                              accumulate);
-        return;
-    }
     using Rec = Record<STORE>;
     const bool in_image = (p < width) && (q < height);
     RayState R;
-    setup_ray<SMEM>(R, vol, V, B, p, q, in_image, V.win_lo, V.win_hi, tab);
-    AxisState (&ax)[3] = R.ax;
-    bool &alive = R.alive;
-    float &s_cur = R.s_cur;
-    long long &u_cur = R.u_cur;
+    setup_ray(R, vol, V, B, p, q, in_image, V.win_lo, V.win_hi, tab);
+    bool alive = R.alive;
+    float s_cur = R.s_cur;
+    long long u_cur = R.u_cur;
+    const float s_lim = march_end(R, V.kk_hi);
     const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
     const long long du0 = V.du[0], du1 = V.du[1], du2 = V.du[2];
-#ifdef GBD_CHECKED
-    int (&kc)[3] = R.kc;
-    const int kd0 = R.kd[0], kd1 = R.kd[1], kd2 = R.kd[2];
-#endif
-    const int Mm1 = vol.M - 1;
-
+    const int M = vol.M;
     BoostConsts bc;
     bc.shx = V.sh_hi[0]; bc.shy = V.sh_hi[1]; bc.shz = V.sh_hi[2];
     bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
     bc.expo = V.expo;
     bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-
-    const long long es = vol.epoch_stride;
-    const void *recs = vol.rec;
-    // Paired float32 records: a sample that reads no snapshot loads the zero
-    // record pair after the last block instead of skipping its loads (faster
-    // for the 32-byte pairs; for 16-byte pairs it costs registers and time).
-    constexpr bool kZeroPair = PAIRED && NCH == 0 && !TOUCH && STORE == GBD_STORE_F32;
-    const long long zero_off = static_cast<long long>(vol.M + 1) * es;
+    bc.plain = false;
+    // blocks and records as in march_ray_bf16.  Paired float32: a sample that
+    // reads no snapshot loads the zero record pair after the last block
+    // (faster for 32-byte pairs than a predicated load).
+    constexpr unsigned kRec = STORE == GBD_STORE_F32 ? 16 : 8;
+    constexpr unsigned kUnit = PAIRED ? 2 * kRec : kRec;
+    constexpr bool kZeroPair = PAIRED && STORE == GBD_STORE_F32;
+    const long long es_bytes = vol.epoch_stride * kRec;
+    const unsigned long long recb = reinterpret_cast<unsigned long long>(vol.rec);
+    const unsigned long long base = recb - (PAIRED ? 0 : es_bytes);
+    const unsigned long long zero_addr = recb + static_cast<unsigned long long>((vol.M + 1) * es_bytes);
 
     float acc = 0.f, comp = 0.f;
     uint32_t count = 0;
-    float cacc[NCH > 0 ? NCH : 1], ccomp[NCH > 0 ? NCH : 1];
+    constexpr int kNch = NCH > 0 ? NCH : 1;
+    float cacc[kNch], ccomp[kNch];
 #pragma unroll
-    for (int c = 0; c < (NCH > 0 ? NCH : 1); ++c) cacc[c] = ccomp[c] = 0.f;
+    for (int c = 0; c < kNch; ++c) cacc[c] = ccomp[c] = 0.f;
 
-    // ---------------- the march, float32 per cell ----------------
-    // Per cell: the nearest face, the chord from the previous exit, the epoch
-    // coordinate at the chord midpoint, and one step of the exit axis.  The
-    // ray ends past the last time that reaches a snapshot or at a sentinel.
-    while (__any_sync(kFull, alive)) {
-        long long off[DEPTH];
-        long long coff[DEPTH];  // channel offset (vector renders)
-        float wgt[DEPTH], dsv[DEPTH];
-        bool has_lo[DEPTH], has_hi[DEPTH];
+    constexpr int H = DEPTH > 1 ? DEPTH / 2 : 1;  // cells per stage (see run_stages)
+    struct Stage {
+        float wgt[H], dsv[H];
+        bool has[H];
+        typename Rec::T rlo[H], rhi[H];
+        float clo[H][kNch], chi[H][kNch];
+    };
+    auto gather = [&](Stage &T) {
 #pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
-            has_lo[d] = false;
-            has_hi[d] = false;
-            off[d] = kZeroPair ? zero_off : 0;
-            coff[d] = 0;
-            wgt[d] = 0.f;
-            dsv[d] = 0.f;
-            if (alive) {
-                // The cell is left through the nearest face; ties go to the
-                // lowest axis (the zero-length chord that follows adds nothing).
-                const bool x0 = ax[0].sn <= ax[1].sn && ax[0].sn <= ax[2].sn;
-                const bool x1 = !x0 && ax[1].sn <= ax[2].sn;
-                const float s_exit = x0 ? ax[0].sn : (x1 ? ax[1].sn : ax[2].sn);
-                const long long u_exit = x0 ? ax[0].un : (x1 ? ax[1].un : ax[2].un);
-                const float ds = s_exit - s_cur;
-                // epoch coordinate at the chord midpoint: m_bar + w, w in [0, 1)
-                const long long um = (u_cur + u_exit) >> 1;
-                const int mb = static_cast<int>(um >> 32);
-                const uint32_t frac = static_cast<uint32_t>(um);
-                const float w = static_cast<float>(frac) * 2.3283064365386963e-10f;
-                // -1 <= m_bar <= M - 1 (at u = -1 exactly both weights vanish below)
-                const bool inside = static_cast<unsigned>(mb + 1) <= static_cast<unsigned>(Mm1 + 1);
-                if (ds > 0.f && inside) {
-                    has_lo[d] = mb >= 0;
-                    has_hi[d] = (mb < Mm1) && (frac != 0u);
+        for (int d = 0; d < H; ++d) {
+            const ExitFace X = exit_face(R.ax, alive);
+            const long long u_exit = X.x0 ? R.ax[0].un : (X.x1 ? R.ax[1].un : R.ax[2].un);
+            const float ds = X.s - s_cur;
+            // epoch coordinate at the chord midpoint: m_bar + w, w in [0, 1)
+            const long long um = (u_cur + u_exit) >> 1;
+            const int bp = static_cast<int>(um >> 32) + 1;
+            const uint32_t frac = static_cast<uint32_t>(um);
+            // -1 <= m_bar <= M - 1 (at u = -1 exactly both weights vanish)
+            const bool take = alive & (ds > 0.f) & (static_cast<unsigned>(bp) <= static_cast<unsigned>(M));
+            bool has_lo = take & (bp != 0);
+            bool has_hi = take & (bp < M) & (frac != 0u);
 #ifdef GBD_CHECKED
-                    if ((has_lo[d] && !check_cell(vol, err_word, kc[0], kc[1], kc[2], mb)) ||
-                        (has_hi[d] && !check_cell(vol, err_word, kc[0], kc[1], kc[2], mb + 1))) {
-                        has_lo[d] = has_hi[d] = false;
-                    }
+            if ((has_lo && !check_cell(vol, err_word, R.kc[0], R.kc[1], R.kc[2], bp - 1)) ||
+                (has_hi && !check_cell(vol, err_word, R.kc[0], R.kc[1], R.kc[2], bp)))
+                has_lo = has_hi = false;
 #endif
-                    const int sum = ax[0].o + ax[1].o + ax[2].o;
-                    // unpaired: snapshot m at block m; paired: snapshots mb and
-                    // mb + 1 side by side in block mb + 1
-                    if (!kZeroPair || has_lo[d] || has_hi[d])
-                        off[d] = PAIRED ? static_cast<long long>(mb + 1) * es + 2LL * sum
-                                        : static_cast<long long>(mb) * es + sum;
-                    if constexpr (NCH > 0 || TOUCH) coff[d] = static_cast<long long>(mb) * ch.cell_stride + sum;
-                    wgt[d] = w;
-                    dsv[d] = ds;
-                }
-                step_exit<SMEM>(ax, x0, x1, ia0, ia1, ia2, du0, du1, du2, tab);
-#ifdef GBD_CHECKED
-                kc[0] += x0 ? kd0 : 0;
-                kc[1] += x1 ? kd1 : 0;
-                kc[2] += (!x0 && !x1) ? kd2 : 0;
-#endif
-                s_cur = s_exit;
-                u_cur = u_exit;
-                // Past the last time that reaches a snapshot (u < -1: the high
-                // word below -1; at u = -1 exactly one more empty step), or out
-                // of the box: nothing further along the ray can contribute.
-                alive = static_cast<int>(u_exit >> 32) >= -1 && (ax[0].o | ax[1].o | ax[2].o) >= 0;
-            }
-        }
-        typename Rec::T rlo[DEPTH], rhi[DEPTH];
-#pragma unroll
-        for (int d = 0; d < DEPTH; ++d) {
+            T.wgt[d] = static_cast<float>(frac) * 2.3283064365386963e-10f;
+            T.dsv[d] = ds;
+            T.has[d] = has_lo | has_hi;
             if constexpr (TOUCH) {
-                rlo[d] = Rec::zero();
-                rhi[d] = Rec::zero();
-                if (has_lo[d]) atomicOr(ch.touch + (coff[d] >> 5), 1u << (coff[d] & 31));
-                if (has_hi[d]) {
-                    const long long i = coff[d] + ch.cell_stride;
+                const long long bit = static_cast<long long>(bp - 1) * ch.cell_stride + R.sum;
+                if (has_lo) atomicOr(ch.touch + (bit >> 5), 1u << (bit & 31));
+                if (has_hi) {
+                    const long long i = bit + ch.cell_stride;
                     atomicOr(ch.touch + (i >> 5), 1u << (i & 31));
                 }
-            } else if (kZeroPair) {
-                Rec::load_pair(recs, off[d], rlo[d], rhi[d]);  // the zero pair when it reads no snapshot
-            } else if (PAIRED) {
-                rlo[d] = Rec::zero();
-                rhi[d] = Rec::zero();
-                if (has_lo[d] || has_hi[d]) Rec::load_pair(recs, off[d], rlo[d], rhi[d]);
             } else {
-                rlo[d] = has_lo[d] ? Rec::load(recs, off[d]) : Rec::zero();
-                rhi[d] = has_hi[d] ? Rec::load(recs, off[d] + es) : Rec::zero();
-            }
-        }
-        float clo[DEPTH][NCH > 0 ? NCH : 1], chi[DEPTH][NCH > 0 ? NCH : 1];
-        if constexpr (NCH > 0) {
-#pragma unroll
-            for (int d = 0; d < DEPTH; ++d)
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    const float *base = ch.chan + c * ch.comp_stride + coff[d];
-                    clo[d][c] = has_lo[d] ? __ldg(base) : 0.f;
-                    chi[d][c] = has_hi[d] ? __ldg(base + ch.cell_stride) : 0.f;
-                }
-        }
-        if constexpr (NCH == 0) {
-            // A snapshot that a sample does not read is a zero record (not
-            // loaded, or the zero record beside the first and the last
-            // snapshot of a paired layout), whose boosted value is exactly 0,
-            // so both are evaluated without a branch.  The compensated sum
-            // takes a sample only where it read a snapshot, so a ray's sum
-            // does not depend on how long the other lanes of its warp march.
-#pragma unroll
-            for (int d = 0; d < DEPTH; ++d) {
-                float vlo, vhi;
-                if constexpr (STORE == GBD_STORE_F32) {
-                    // per record (the lone march measured faster this way)
-                    vlo = Rec::boosted(rlo[d], bc);
-                    vhi = Rec::boosted(rhi[d], bc);
+                const unsigned long long a = rec_addr<kUnit>(base, bp, es_bytes, R.sum);
+                if constexpr (kZeroPair) {
+                    const unsigned long long pa = T.has[d] ? a : zero_addr;
+                    T.rlo[d] = Rec::load_at(pa);
+                    T.rhi[d] = Rec::load_at(pa + kRec);
+                } else if constexpr (PAIRED) {
+                    T.rlo[d] = Rec::zero();
+                    T.rhi[d] = Rec::zero();
+                    if (has_lo | has_hi) Rec::load_pair_at(a, T.rlo[d], T.rhi[d]);
                 } else {
-                    const float2 vv = Rec::boosted2(rlo[d], rhi[d], bc);
-                    vlo = vv.x;
-                    vhi = vv.y;
+                    T.rlo[d] = has_lo ? Rec::load_at(a) : Rec::zero();
+                    T.rhi[d] = has_hi ? Rec::load_at(a + es_bytes) : Rec::zero();
                 }
-                const float v = fmaf(wgt[d], vhi - vlo, vlo);       // Eq. 8
-                const float y = fmaf(v, dsv[d], -comp);             // compensated sum
-                const float t = acc + y;
-                const bool take = has_lo[d] || has_hi[d];
-                comp = take ? (t - acc) - y : comp;
-                acc = take ? t : acc;
-                count += take ? 1u : 0u;
             }
-        } else {
-            // vector renders: the Doppler factor of each snapshot serves every channel
+            if constexpr (NCH > 0) {
+                const float *cp = ch.chan + (static_cast<long long>(bp - 1) * ch.cell_stride + R.sum);
 #pragma unroll
-            for (int d = 0; d < DEPTH; ++d) {
-                if (!(has_lo[d] || has_hi[d])) continue;
-                const float blo = has_lo[d] ? Rec::boost(rlo[d], bc) : 0.f;
-                const float bhi = has_hi[d] ? Rec::boost(rhi[d], bc) : 0.f;
-                const float vlo = has_lo[d] ? Rec::emissivity(rlo[d]) * blo : 0.f;
-                const float vhi = has_hi[d] ? Rec::emissivity(rhi[d]) * bhi : 0.f;
-                const float v = fmaf(wgt[d], vhi - vlo, vlo);
-                const float y = fmaf(v, dsv[d], -comp);
-                const float t = acc + y;
-                comp = (t - acc) - y;
-                acc = t;
+                for (int c = 0; c < NCH; ++c, cp += ch.comp_stride) {
+                    T.clo[d][c] = has_lo ? __ldg(cp) : 0.f;
+                    T.chi[d][c] = has_hi ? __ldg(cp + ch.cell_stride) : 0.f;
+                }
+            }
+            step_exact(R, X, ia0, ia1, ia2, du0, du1, du2, tab);
+            s_cur = X.s;
+            u_cur = u_exit;
+            alive = alive & (X.s < s_lim);
+        }
+    };
+    // A snapshot the sample does not read is a zero record (boosted value
+    // exactly 0); the compensated sums take the sample only where it read
+    // one, so a ray's sum does not depend on how long the other lanes of
+    // its warp march.
+    auto evaluate = [&](const Stage &T) {
+        if constexpr (TOUCH) return;
+#pragma unroll
+        for (int d = 0; d < H; ++d) {
+            const bool take = T.has[d];
+            const float blo = Rec::boost(T.rlo[d], bc), bhi = Rec::boost(T.rhi[d], bc);
+            const float vlo = __fmul_rn(Rec::emissivity(T.rlo[d]), blo);
+            const float v = fmaf(T.wgt[d], fmaf(Rec::emissivity(T.rhi[d]), bhi, -vlo), vlo);  // Eq. 8
+            const float y = fmaf(v, T.dsv[d], -comp);
+            const float t = acc + y;
+            comp = take ? (t - acc) - y : comp;
+            acc = take ? t : acc;
+            count += take ? 1u : 0u;
+            if constexpr (NCH > 0) {
+                // the Doppler factor of each snapshot serves every channel
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
-                    const float ulo = clo[d][c] * blo, uhi = chi[d][c] * bhi;
-                    const float u = fmaf(wgt[d], uhi - ulo, ulo);
-                    const float yc = fmaf(u, dsv[d], -ccomp[c]);
+                    const float ulo = T.clo[d][c] * blo, uhi = T.chi[d][c] * bhi;
+                    const float u = fmaf(T.wgt[d], uhi - ulo, ulo);
+                    const float yc = fmaf(u, T.dsv[d], -ccomp[c]);
                     const float tc = cacc[c] + yc;
-                    ccomp[c] = (tc - cacc[c]) - yc;
-                    cacc[c] = tc;
+                    ccomp[c] = take ? (tc - cacc[c]) - yc : ccomp[c];
+                    cacc[c] = take ? tc : cacc[c];
                 }
-                ++count;
             }
         }
-    }
-
+    };
+    run_stages<(DEPTH > 1), Stage>(alive, gather, evaluate);
     if (in_image && !TOUCH) {
         const long long pix = static_cast<long long>(q) * width + p;
         if (PARTIAL) {
@@ -1046,265 +866,22 @@ __device__ __forceinline__ void march_ray(const VolDev &vol, const ViewDev &V, c
     }
 }
 
-// march_group for bfloat16/float16 records, with the float epoch coordinate
-// of the bfloat16/float16 march (EpochLine of the reference member) and the
-// step without branches.  Member g's coordinate at a chord midpoint is the
-// reference member's plus dlf[g] = Delta_g rounded to float.  GD cells are
-// traversed per iteration; then each member gathers its records of all GD
-// cells before evaluating them, so a member keeps GD loads in flight.
-template <bool PAIRED, int G, bool PLAIN, int GD>
-__device__ __forceinline__ void march_group_bf16(const VolDev &vol, const ViewDev &V, float win_lo, float win_hi,
-                                                 const ViewDev *GV, const long long *dl, const int *dh, int gcnt,
-                                                 const RayBox &B, int p, int q, int width, int height, float *out,
-                                                 long long img_stride, uint32_t *cnt_img, int *err_word,
-                                                 const int32_t *__restrict__ tab)
+template <int STORE, int DEPTH, bool PAIRED, bool PARTIAL = false, int NCH = 0, bool TOUCH = false>
+__device__ __forceinline__ void march_ray(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
+                                          int width, int height, float *out_img, uint32_t *cnt_img, int *err_word,
+                                          const int32_t *__restrict__ tab, bool accumulate = false,
+                                          const ChanPtrs ch = ChanPtrs{nullptr, 0, 0, nullptr})
 {
-    using Rec = Record<GBD_STORE_BF16_F16U>;
-    const bool in_image = (p < width) && (q < height);
-    RayState R;
-    setup_ray<true>(R, vol, V, B, p, q, in_image, win_lo, win_hi, tab);
-    AxisState (&ax)[3] = R.ax;
-    bool alive = R.alive;
-    float s_cur = R.s_cur;
-    const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
-    const EpochLine L = epoch_line(R, V);
-    const int M = vol.M;
-#ifdef GBD_CHECKED
-    int (&kc)[3] = R.kc;
-    const int kd0 = R.kd[0], kd1 = R.kd[1], kd2 = R.kd[2];
-#endif
-
-    BoostConsts bc;
-    bc.shx = V.sh_hi[0]; bc.shy = V.sh_hi[1]; bc.shz = V.sh_hi[2];
-    bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
-    bc.expo = V.expo;
-    bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-    bc.plain = PLAIN;
-    constexpr unsigned long long kUnit = PAIRED ? 16ull : 8ull;
-    const unsigned long long recb = reinterpret_cast<unsigned long long>(vol.rec);
-    const long long es_bytes = vol.epoch_stride * 8LL;
-
-    float dlf[G];
-    float acc[G];
-    uint32_t count[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        dlf[g] = g < gcnt ? fix_to_float(dl[g], 1.0f / kTwo32) : 0.f;
-        acc[g] = 0.f;
-        count[g] = 0u;
-    }
-
-    while (__any_sync(kFull, alive)) {
-        float umv[GD], dsv[GD];  // reference member's epoch coordinate at the chord midpoints, chords
-        int smv[GD];             // layout offsets of the cells
-        bool posv[GD];           // positive chords
-#ifdef GBD_CHECKED
-        int kcs[GD][3];
-#endif
-        int mlo = INT_MAX, mhi = INT_MIN;  // the warp's range of reference snapshot indices
-#pragma unroll
-        for (int d = 0; d < GD; ++d) {
-            const bool x0 = alive && ax[0].sn <= ax[1].sn && ax[0].sn <= ax[2].sn;
-            const bool x1 = alive && !x0 && ax[1].sn <= ax[2].sn;
-            const bool x2 = alive && !x0 && !x1;
-            const float s_exit = x0 ? ax[0].sn : (x1 ? ax[1].sn : ax[2].sn);
-            dsv[d] = s_exit - s_cur;
-            umv[d] = fmaf(L.mkk, s_cur + s_exit, L.c0);
-            posv[d] = alive && dsv[d] > 0.f;
-            smv[d] = ax[0].o + ax[1].o + ax[2].o;
-            const int mref = static_cast<int>(floorf(umv[d]));
-            mlo = posv[d] ? min(mlo, mref) : mlo;
-            mhi = posv[d] ? max(mhi, mref) : mhi;
-#ifdef GBD_CHECKED
-            kcs[d][0] = kc[0];
-            kcs[d][1] = kc[1];
-            kcs[d][2] = kc[2];
-            kc[0] += x0 ? kd0 : 0;
-            kc[1] += x1 ? kd1 : 0;
-            kc[2] += x2 ? kd2 : 0;
-#endif
-            step_lite<true>(ax, x0, x1, x2, ia0, ia1, ia2, tab);
-            s_cur = s_exit;
-            alive = alive && s_exit <= L.s_stop && (ax[0].o | ax[1].o | ax[2].o) >= 0;
-        }
-        mlo = __reduce_min_sync(kFull, mlo);
-        mhi = __reduce_max_sync(kFull, mhi);
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            // Member g's snapshot index at a midpoint is mref + dh[g] or one
-            // more: skip it when no lane of the warp can reach [-1, M - 1].
-            if (g >= gcnt || mlo > mhi || static_cast<long long>(mhi) + dh[g] < -2 ||
-                static_cast<long long>(mlo) + dh[g] > M - 1)
-                continue;
-            typename Rec::T rlo[GD], rhi[GD];
-            float wg[GD];
-            bool tk[GD];
-#pragma unroll
-            for (int d = 0; d < GD; ++d) {
-                const float ug = umv[d] + dlf[g];
-                const float fl = floorf(ug);
-                const float w = ug - fl;
-                const int mb = static_cast<int>(fl);
-                const bool take = posv[d] && static_cast<unsigned>(mb + 1) <= static_cast<unsigned>(M);
-                bool has_lo = take && mb >= 0;
-                bool has_hi = take && mb < M - 1 && w != 0.f;
-#ifdef GBD_CHECKED
-                if ((has_lo && !check_cell(vol, err_word, kcs[d][0], kcs[d][1], kcs[d][2], mb)) ||
-                    (has_hi && !check_cell(vol, err_word, kcs[d][0], kcs[d][1], kcs[d][2], mb + 1)))
-                    has_lo = has_hi = false;
-#endif
-                const unsigned long long pa =
-                    recb + static_cast<unsigned long long>(static_cast<long long>(PAIRED ? mb + 1 : mb) * es_bytes) +
-                    static_cast<unsigned long long>(static_cast<uint32_t>(smv[d])) * kUnit;
-                rlo[d] = Rec::zero();
-                rhi[d] = Rec::zero();
-                if (PAIRED) {
-                    if (has_lo || has_hi) Rec::load_pair_at(pa, rlo[d], rhi[d]);
-                } else {
-                    if (has_lo) rlo[d] = Rec::load_at(pa);
-                    if (has_hi) rhi[d] = Rec::load_at(pa + es_bytes);
-                }
-                wg[d] = take ? w : 0.f;
-                tk[d] = has_lo || has_hi;
-            }
-#pragma unroll
-            for (int d = 0; d < GD; ++d) {
-                const float2 vv = PLAIN ? Rec::boosted2_plain(rlo[d], rhi[d], bc) : Rec::boosted2(rlo[d], rhi[d], bc);
-                const float v = fmaf(wg[d], vv.y - vv.x, vv.x);  // Eq. 8
-                acc[g] = fmaf(v, posv[d] ? dsv[d] : 0.f, acc[g]);
-                count[g] += tk[d] ? 1u : 0u;
-            }
-        }
-    }
-
-    if (in_image) {
-        const long long pix = static_cast<long long>(q) * width + p;
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            if (g >= gcnt) break;
-            out[g * img_stride + pix] = GV[g].prefactor * acc[g];
-            if (cnt_img) cnt_img[g * img_stride + pix] = count[g];
-        }
-    }
-}
-
-// march_group for float32 records without branches (the step of
-// march_ray_f32), exact epoch coordinate and compensated sums.  Each member's
-// arithmetic is that of the branching form, value for value.
-template <bool PAIRED, int G>
-__device__ __forceinline__ void march_group_f32(const VolDev &vol, const ViewDev &V, float win_lo, float win_hi,
-                                                const ViewDev *GV, const long long *dl, const int *dh, int gcnt,
-                                                const RayBox &B, int p, int q, int width, int height, float *out,
-                                                long long img_stride, uint32_t *cnt_img, int *err_word,
-                                                const int32_t *__restrict__ tab)
-{
-    using Rec = Record<GBD_STORE_F32>;
-    const bool in_image = (p < width) && (q < height);
-    RayState R;
-    setup_ray<true>(R, vol, V, B, p, q, in_image, win_lo, win_hi, tab);
-    AxisState (&ax)[3] = R.ax;
-    bool alive = R.alive;
-    float s_cur = R.s_cur;
-    long long u_cur = R.u_cur;
-    const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
-    const long long du0 = V.du[0], du1 = V.du[1], du2 = V.du[2];
-    const int Mm1 = vol.M - 1;
-#ifdef GBD_CHECKED
-    int (&kc)[3] = R.kc;
-    const int kd0 = R.kd[0], kd1 = R.kd[1], kd2 = R.kd[2];
-#endif
-    BoostConsts bc;
-    bc.shx = V.sh_hi[0]; bc.shy = V.sh_hi[1]; bc.shz = V.sh_hi[2];
-    bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
-    bc.expo = V.expo;
-    bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-    bc.plain = false;
-    constexpr unsigned long long kUnit = PAIRED ? 32ull : 16ull;
-    const unsigned long long recb = reinterpret_cast<unsigned long long>(vol.rec);
-    const long long es_bytes = vol.epoch_stride * 16LL;
-    const unsigned long long zero_addr = recb + static_cast<unsigned long long>((vol.M + 1) * es_bytes);
-
-    float acc[G], comp[G];
-    uint32_t count[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-        acc[g] = comp[g] = 0.f;
-        count[g] = 0u;
-    }
-
-    while (__any_sync(kFull, alive)) {
-        const bool x0 = alive && ax[0].sn <= ax[1].sn && ax[0].sn <= ax[2].sn;
-        const bool x1 = alive && !x0 && ax[1].sn <= ax[2].sn;
-        const bool x2 = alive && !x0 && !x1;
-        const float s_exit = x0 ? ax[0].sn : (x1 ? ax[1].sn : ax[2].sn);
-        const long long u_exit = x0 ? ax[0].un : (x1 ? ax[1].un : ax[2].un);
-        const float ds = s_exit - s_cur;
-        const long long um = (u_cur + u_exit) >> 1;  // reference epoch coordinate at the chord midpoint
-        const bool pos = alive && ds > 0.f;
-        const int sm = ax[0].o + ax[1].o + ax[2].o;
-        const int mref = static_cast<int>(um >> 32);
-        const int mlo = __reduce_min_sync(kFull, pos ? mref : INT_MAX);
-        const int mhi = __reduce_max_sync(kFull, pos ? mref : INT_MIN);
-#ifdef GBD_CHECKED
-        const int kc0 = kc[0], kc1 = kc[1], kc2 = kc[2];
-        kc[0] += x0 ? kd0 : 0;
-        kc[1] += x1 ? kd1 : 0;
-        kc[2] += x2 ? kd2 : 0;
-#endif
-        step_nb<true>(ax, x0, x1, x2, ia0, ia1, ia2, du0, du1, du2, tab);
-        s_cur = s_exit;
-        u_cur = u_exit;
-        alive = alive && static_cast<int>(u_exit >> 32) >= -1 && (ax[0].o | ax[1].o | ax[2].o) >= 0;
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            // Member g's snapshot index at a midpoint is mref + dh[g] or one
-            // more: skip it when no lane of the warp can reach [-1, M - 1].
-            if (g >= gcnt || mlo > mhi || static_cast<long long>(mhi) + dh[g] < -2 ||
-                static_cast<long long>(mlo) + dh[g] > Mm1)
-                continue;
-            const long long ug = um + dl[g];
-            const int mb = static_cast<int>(ug >> 32);
-            const uint32_t frac = static_cast<uint32_t>(ug);
-            const float w = static_cast<float>(frac) * 2.3283064365386963e-10f;
-            const bool take = pos && static_cast<unsigned>(mb + 1) <= static_cast<unsigned>(Mm1 + 1);
-            bool has_lo = take && mb >= 0;
-            bool has_hi = take && mb < Mm1 && frac != 0u;
-#ifdef GBD_CHECKED
-            if ((has_lo && !check_cell(vol, err_word, kc0, kc1, kc2, mb)) ||
-                (has_hi && !check_cell(vol, err_word, kc0, kc1, kc2, mb + 1)))
-                has_lo = has_hi = false;
-#endif
-            const unsigned long long a =
-                recb + static_cast<unsigned long long>(static_cast<long long>(PAIRED ? mb + 1 : mb) * es_bytes) +
-                static_cast<unsigned long long>(static_cast<uint32_t>(sm)) * kUnit;
-            typename Rec::T rlo, rhi;
-            if (PAIRED) {
-                const float4 *ptr = reinterpret_cast<const float4 *>((has_lo || has_hi) ? a : zero_addr);
-                rlo = __ldg(ptr);
-                rhi = __ldg(ptr + 1);
-            } else {
-                rlo = has_lo ? __ldg(reinterpret_cast<const float4 *>(a)) : Rec::zero();
-                rhi = has_hi ? __ldg(reinterpret_cast<const float4 *>(a + es_bytes)) : Rec::zero();
-            }
-            const float vlo = Rec::boosted(rlo, bc), vhi = Rec::boosted(rhi, bc);
-            const float v = fmaf(w, vhi - vlo, vlo);     // Eq. 8
-            const float y = fmaf(v, ds, -comp[g]);       // compensated sum
-            const float t = acc[g] + y;
-            const bool tk = has_lo || has_hi;
-            comp[g] = tk ? (t - acc[g]) - y : comp[g];
-            acc[g] = tk ? t : acc[g];
-            count[g] += tk ? 1u : 0u;
-        }
-    }
-
-    if (in_image) {
-        const long long pix = static_cast<long long>(q) * width + p;
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-            if (g >= gcnt) break;
-            out[g * img_stride + pix] = GV[g].prefactor * acc[g];
-            if (cnt_img) cnt_img[g * img_stride + pix] = count[g];
-        }
+    if constexpr (STORE == GBD_STORE_BF16_F16U && NCH == 0 && !TOUCH) {
+        if (vol.plain_boost)
+            march_ray_bf16<DEPTH, PAIRED, PARTIAL, true>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
+                                                         tab, accumulate);
+        else
+            march_ray_bf16<DEPTH, PAIRED, PARTIAL, false>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
+                                                          tab, accumulate);
+    } else {
+        march_ray_exact<STORE, DEPTH, PAIRED, PARTIAL, NCH, TOUCH>(vol, V, B, p, q, width, height, out_img, cnt_img,
+                                                                   err_word, tab, accumulate, ch);
     }
 }
 
@@ -1314,34 +891,203 @@ __device__ __forceinline__ void march_group_f32(const VolDev &vol, const ViewDev
 // members' windows and carries the epoch coordinate of the reference member,
 // the one whose window ends last (largest u_obs); member g's coordinate
 // differs from it by the exact constant Delta_g = u_obs,g - u_obs,ref <= 0
-// (Q31.32), so at a chord midpoint it is um + Delta_g.  Per cell the
-// traversal is done once, and every member whose window some lane of the warp
-// reaches gathers, boosts and sums its own two snapshots into its own
-// compensated sum (Eq. 19 per view).  A member's pixel is summed over the same
-// cells, chords and midpoints as when its view is marched alone; the crossings
-// are measured from the group's anchor instead of the view's own, so the two
-// agree to float rounding, not bit for bit.  Member g's image is at
-// out + g * img_stride.
-template <int STORE, int DEPTH, bool PAIRED, int G>
+// (Q31.32), so at a chord midpoint it is um + Delta_g.
+//
+// The members also share the snapshots.  Their coordinates lie within S - 2
+// snapshots of each other (the host's grouping rule), so the two snapshots
+// that any member interpolates between are among the S from the reference's
+// upper one, m_0 = floor(um) + 1, down to m_0 - S + 1.  Per cell those S records
+// are gathered and boosted once, and each member only picks its pair, forms
+// its hat weight and adds to its own sum (Eq. 19 per view).  Snapshots that no
+// member of the lane reaches are not read.
+//
+// What bounds it: instruction issue, as for the lone march.  A cell costs the
+// traversal once, S records of about 16 (float32) or 8 (bfloat16/float16)
+// instructions of boost, and about 18 or 13 per member, where the members once
+// gathered and boosted two records each (18 images of 512^2 of a 256^3 x 16
+// series, groups of three: float32 892 -> 580 us, bfloat16/float16 600 -> 428).
+//
+// A member's pixel is summed over the same cells, chords, midpoints and
+// boosted values as when its view is marched alone; the crossings are measured
+// from the group's anchor instead of the view's own, so the two agree to float
+// rounding, not bit for bit.  Member g's image is at out + g * img_stride.
+// GD cells are traversed per iteration, and all their records gathered before
+// any is evaluated.
+template <int STORE, int GD, int G, int S, bool PLAIN>
 __device__ __forceinline__ void march_group(const VolDev &vol, const ViewDev &V, float win_lo, float win_hi,
-                                            const ViewDev *GV, const long long *dl, const int *dh, int gcnt,
-                                            const RayBox &B, int p, int q, int width, int height, float *out,
-                                            long long img_stride, uint32_t *cnt_img, int *err_word,
-                                            const int32_t *__restrict__ tab)
+                                            const ViewDev *GV, const long long *dl, int gcnt, const RayBox &B, int p,
+                                            int q, int width, int height, float *out, long long img_stride,
+                                            uint32_t *cnt_img, int *err_word, const int32_t *__restrict__ tab)
 {
-    if constexpr (STORE == GBD_STORE_F32) {
-        march_group_f32<PAIRED, G>(vol, V, win_lo, win_hi, GV, dl, dh, gcnt, B, p, q, width, height, out, img_stride,
-                                   cnt_img, err_word, tab);
-        return;
+    constexpr bool kF32 = STORE == GBD_STORE_F32;
+    using Rec = Record<STORE>;
+    const bool in_image = (p < width) && (q < height);
+    RayState R;
+    setup_ray(R, vol, V, B, p, q, in_image, win_lo, win_hi, tab);
+    bool alive = R.alive;
+    float s_cur = R.s_cur;
+    long long u_cur = R.u_cur;
+    const float ia0 = V.inv_a[0], ia1 = V.inv_a[1], ia2 = V.inv_a[2];
+    const long long du0 = V.du[0], du1 = V.du[1], du2 = V.du[2];
+    const EpochLine L = epoch_line(R, V);
+    const float s_lim = kF32 ? march_end(R, V.kk_hi) : L.s_lim;
+    const int M = vol.M;
+
+    BoostConsts bc;
+    bc.shx = V.sh_hi[0]; bc.shy = V.sh_hi[1]; bc.shz = V.sh_hi[2];
+    bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
+    bc.expo = V.expo;
+    bc.beaming = (V.flags & GBD_BEAMING) != 0u;
+    bc.plain = PLAIN;
+
+    // Unpaired, snapshot m is a record of block m.  Paired, block m holds the
+    // records of m - 1 and m side by side: of the snapshots m_0 - k, the even k
+    // are the second records of blocks m_0 - k and the odd k the first ones of
+    // blocks m_0 - k + 1, so that neighbours share a sector.  Either way the record of
+    // m_0 - k lies (k & 1) odd_bytes + (k & ~1) blk_bytes below that of m_0.
+    constexpr unsigned kRec = kF32 ? 16 : 8;
+    const long long blk_bytes = vol.epoch_stride * kRec;
+    const long long odd_bytes = vol.paired ? kRec : blk_bytes;
+    const int cell_shift = vol.paired ? 1 : 0;
+    const unsigned long long recb = reinterpret_cast<unsigned long long>(vol.rec) + (vol.paired ? kRec : 0u);
+
+    float dlf[G];  // Delta_g as a float (bfloat16/float16 march)
+    float acc[G], comp[G];
+    uint32_t count[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        dlf[g] = (!kF32 && g < gcnt) ? fix_to_float(dl[g], 1.0f / kTwo32) : 0.f;
+        acc[g] = comp[g] = 0.f;
+        count[g] = 0u;
     }
-    if constexpr (STORE == GBD_STORE_BF16_F16U) {
-        if (vol.plain_boost)
-            march_group_bf16<PAIRED, G, true, DEPTH>(vol, V, win_lo, win_hi, GV, dl, dh, gcnt, B, p, q, width, height,
-                                                     out, img_stride, cnt_img, err_word, tab);
-        else
-            march_group_bf16<PAIRED, G, false, DEPTH>(vol, V, win_lo, win_hi, GV, dl, dh, gcnt, B, p, q, width, height,
-                                                      out, img_stride, cnt_img, err_word, tab);
-        return;
+    long long dl_min = 0;  // the earliest member's
+    for (int g = 0; g < gcnt; ++g) dl_min = min(dl_min, dl[g]);
+    const float dlf_min = fix_to_float(dl_min, 1.0f / kTwo32);
+
+    while (__any_sync(kFull, alive)) {
+        long long umx[GD];          // the reference's epoch coordinate at the chord midpoints (float32 march)
+        float umf[GD], dsv[GD];     // the same (bfloat16/float16 march), and the chords (0 where there is none)
+        typename Rec::T rec[GD][S];  // snapshots m_0, m_0 - 1, ... of each cell
+        bool pos[GD];
+#pragma unroll
+        for (int d = 0; d < GD; ++d) {
+            const ExitFace X = exit_face(R.ax, alive);
+            const float ds = X.s - s_cur;
+            pos[d] = alive && ds > 0.f;
+            dsv[d] = pos[d] ? ds : 0.f;
+            int top, low;  // m_0, and the lowest snapshot that a member reaches
+            long long u_exit = 0;
+            if constexpr (kF32) {
+                u_exit = X.x0 ? R.ax[0].un : (X.x1 ? R.ax[1].un : R.ax[2].un);
+                umx[d] = (u_cur + u_exit) >> 1;
+                top = static_cast<int>(umx[d] >> 32) + 1;
+                low = static_cast<int>((umx[d] + dl_min) >> 32);
+            } else {
+                umf[d] = fmaf(L.mkk, s_cur + X.s, L.c0);
+                top = static_cast<int>(floorf(umf[d])) + 1;
+                low = static_cast<int>(floorf(umf[d] + dlf_min));
+            }
+            const unsigned long long at = rec_addr<kRec>(recb, top, blk_bytes, R.sum << cell_shift);
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+                const int m = top - k;
+                bool want = pos[d] && static_cast<unsigned>(m) < static_cast<unsigned>(M) && m >= low;
+#ifdef GBD_CHECKED
+                if (want && !check_cell(vol, err_word, R.kc[0], R.kc[1], R.kc[2], m)) want = false;
+#endif
+                rec[d][k] = Rec::zero();
+                if (want) rec[d][k] = Rec::load_at(at - static_cast<unsigned long long>((k & 1) * odd_bytes + (k & ~1) * blk_bytes));
+            }
+            if constexpr (kF32) {
+                step_exact(R, X, ia0, ia1, ia2, du0, du1, du2, tab);
+                u_cur = u_exit;
+            } else {
+                step_lite(R, X, ia0, ia1, ia2, tab);
+            }
+            s_cur = X.s;
+            alive = alive & (X.s < s_lim);
+        }
+        // boosted value of each snapshot (0 of one not read), and its difference
+        // from the next lower one, as the lone march forms them
+        float b[GD][S], dif[GD][S - 1];
+        if constexpr (kF32) {
+#pragma unroll
+            for (int d = 0; d < GD; ++d) {
+                float bk[S];
+#pragma unroll
+                for (int k = 0; k < S; ++k) {
+                    bk[k] = Rec::boost(rec[d][k], bc);
+                    b[d][k] = __fmul_rn(Rec::emissivity(rec[d][k]), bk[k]);
+                }
+#pragma unroll
+                for (int k = 0; k < S - 1; ++k) dif[d][k] = fmaf(Rec::emissivity(rec[d][k]), bk[k], -b[d][k + 1]);
+            }
+        } else {
+            // two records at a time, over all cells
+#pragma unroll
+            for (int i = 0; i < GD * S; i += 2) {
+                const int d0 = i / S, k0 = i % S, d1 = (i + 1) / S, k1 = (i + 1) % S;
+                const typename Rec::T r1 = i + 1 < GD * S ? rec[d1 < GD ? d1 : 0][k1] : Rec::zero();
+                const float2 vv = PLAIN ? Rec::boosted2_plain(rec[d0][k0], r1, bc) : Rec::boosted2(rec[d0][k0], r1, bc);
+                b[d0][k0] = vv.x;
+                if (i + 1 < GD * S) b[d1 < GD ? d1 : 0][k1] = vv.y;
+            }
+#pragma unroll
+            for (int d = 0; d < GD; ++d)
+#pragma unroll
+                for (int k = 0; k < S - 1; ++k) dif[d][k] = b[d][k] - b[d][k + 1];
+        }
+#pragma unroll
+        for (int d = 0; d < GD; ++d) {
+#pragma unroll
+            for (int g = 0; g < G; ++g) {
+                if (g >= gcnt) break;  // uniform
+                // member g's lower snapshot is m_0 - 1 - k: b[k + 1], its pair's difference dif[k]
+                float w, lower = b[d][1], up = dif[d][0];
+                bool take;
+                if constexpr (kF32) {
+                    const long long ug = umx[d] + dl[g];
+                    const uint32_t frac = static_cast<uint32_t>(ug);
+                    const int mb = static_cast<int>(ug >> 32), m0 = static_cast<int>(umx[d] >> 32);
+                    w = static_cast<float>(frac) * 2.3283064365386963e-10f;
+                    // -1 <= m_bar <= M - 1 (at u = -1 exactly both weights vanish)
+                    take = pos[d] && static_cast<unsigned>(mb + 1) <= static_cast<unsigned>(M) && (mb >= 0 || frac != 0u);
+#pragma unroll
+                    for (int k = 1; k < S - 1; ++k) {
+                        lower = mb <= m0 - k ? b[d][k + 1] : lower;
+                        up = mb <= m0 - k ? dif[d][k] : up;
+                    }
+                    const float v = fmaf(w, up, lower);  // Eq. 8
+                    const float y = fmaf(v, dsv[d], -comp[g]);      // compensated sum
+                    const float t = acc[g] + y;
+                    comp[g] = take ? (t - acc[g]) - y : comp[g];
+                    acc[g] = take ? t : acc[g];
+                } else {
+                    const float ug = umf[d] + dlf[g];
+                    const float fl = floorf(ug), f0 = floorf(umf[d]);
+                    w = ug - fl;
+                    take = pos[d] && fl >= -1.0f && fl <= static_cast<float>(M - 1) && (fl >= 0.f || w != 0.f);
+#pragma unroll
+                    for (int k = 1; k < S - 1; ++k) {
+                        lower = fl <= f0 - static_cast<float>(k) ? b[d][k + 1] : lower;
+                        up = fl <= f0 - static_cast<float>(k) ? dif[d][k] : up;
+                    }
+                    const float v = fmaf(w, up, lower);  // Eq. 8
+                    acc[g] = fmaf(take ? v : 0.f, dsv[d], acc[g]);
+                }
+                count[g] += take ? 1u : 0u;
+            }
+        }
+    }
+
+    if (in_image) {
+        const long long pix = static_cast<long long>(q) * width + p;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            if (g >= gcnt) break;
+            out[g * img_stride + pix] = GV[g].prefactor * acc[g];
+            if (cnt_img) cnt_img[g * img_stride + pix] = count[g];
+        }
     }
 }
 
@@ -1402,7 +1148,7 @@ __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant_
                 const int ty = tile / a.tiles_x;
                 const int p = tx * a.packet_w + lane % a.packet_w;
                 const int q = ty * a.packet_h + lane / a.packet_w;
-                march_ray<STORE, DEPTH, PAIRED, true>(a.vol, V, box, p, q, a.width, a.height, out, cnt,
+                march_ray<STORE, DEPTH, PAIRED>(a.vol, V, box, p, q, a.width, a.height, out, cnt,
                                                       a.error_word, s_tab, a.accumulate != 0);
                 if (!a.persistent) break;
             }
@@ -1424,7 +1170,7 @@ __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant_
             if (a.persistent && a.tile_order) tile = __ldg(a.tile_order + tile);
             const int p = (tile % a.tiles_x) * a.packet_w + lane % a.packet_w;
             const int q = (tile / a.tiles_x) * a.packet_h + lane / a.packet_w;
-            march_ray<STORE, DEPTH, PAIRED, true>(a.vol, V, box, p, q, a.width, a.height, out, cnt, a.error_word,
+            march_ray<STORE, DEPTH, PAIRED>(a.vol, V, box, p, q, a.width, a.height, out, cnt, a.error_word,
                                                   s_tab, a.accumulate != 0);
             if (!a.persistent) break;
         }
@@ -1434,11 +1180,8 @@ __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant_
 // Time groups: march_kernel's work split over groups of views instead of
 // single views (group g is views group_first[g] .. group_first[g + 1] - 1,
 // its CTAs cta_begin[g] .. cta_begin[g + 1] - 1, its tile counter queue[g]).
-// DEPTH cells per iteration for bfloat16/float16 records (each member
-// gathers all of them before evaluating any), one for float32 records, and at
-// most 80 registers: with the compiler's budget (110 - 150) fewer warps fit
-// and the grouped march ran slower than the lone one.
-template <int STORE, int DEPTH, bool PAIRED, int G>
+// DEPTH cells per iteration, S snapshots per cell, at most 80 registers.
+template <int STORE, int DEPTH, int G, int S>
 __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_tab[];
@@ -1484,9 +1227,17 @@ __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ M
             const int ty = tile / a.tiles_x;
             const int p = tx * a.packet_w + lane % a.packet_w;
             const int q = ty * a.packet_h + lane / a.packet_w;
-            march_group<STORE, DEPTH, PAIRED, G>(a.vol, V, win_lo, win_hi, GV, a.view_delta + first,
-                                                 a.view_dhi + first, gcnt, box, p, q, a.width, a.height, out, stride,
-                                                 cnt, a.error_word, s_tab);
+            auto march = [&](auto plain) {
+                march_group<STORE, DEPTH, G, S, decltype(plain)::value>(
+                    a.vol, V, win_lo, win_hi, GV, a.view_delta + first, gcnt, box, p, q, a.width, a.height, out, stride,
+                    cnt, a.error_word, s_tab);
+            };
+            if constexpr (STORE == GBD_STORE_F32) {
+                march(std::false_type{});
+            } else {
+                if (a.vol.plain_boost) march(std::true_type{});
+                else march(std::false_type{});
+            }
             if (!a.persistent) break;
         }
     }
@@ -1533,7 +1284,7 @@ __global__ void __launch_bounds__(256, MINB) vector_kernel(const __grid_constant
             const int ty = tile / a.tiles_x;
             const int p = tx * a.packet_w + lane % a.packet_w;
             const int q = ty * a.packet_h + lane / a.packet_w;
-            march_ray<STORE, 2, PAIRED, true, false, NCH>(a.vol, V, box, p, q, a.width, a.height, out, nullptr,
+            march_ray<STORE, 2, PAIRED, false, NCH>(a.vol, V, box, p, q, a.width, a.height, out, nullptr,
                                                            a.error_word, s_tab, false, ch);
             if (!a.persistent) break;
         }
@@ -1568,7 +1319,7 @@ __global__ void __launch_bounds__(256, 1) touch_kernel(const __grid_constant__ M
     const int q = (tile / a.tiles_x) * a.packet_h + lane / a.packet_w;
     float *out = a.out + static_cast<long long>(vi) * a.width * a.height;
     const ChanPtrs ch{nullptr, 0, cells, bits};
-    march_ray<STORE, 1, PAIRED, true, false, 0, true>(a.vol, V, box, p, q, a.width, a.height, out, nullptr,
+    march_ray<STORE, 1, PAIRED, false, 0, true>(a.vol, V, box, p, q, a.width, a.height, out, nullptr,
                                                        a.error_word, s_tab, false, ch);
 }
 
@@ -1606,24 +1357,24 @@ __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__
     const RayBox box = grid_box(R.vol, R.view);
     if (R.vol.store == GBD_STORE_F32) {
         if (R.vol.paired)
-            march_ray<GBD_STORE_F32, DEPTH, true, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
+            march_ray<GBD_STORE_F32, DEPTH, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
                                                         a.error_word, s_tab);
         else
-            march_ray<GBD_STORE_F32, DEPTH, false, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
+            march_ray<GBD_STORE_F32, DEPTH, false>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
                                                          a.error_word, s_tab);
     } else {
         if (R.vol.paired)
-            march_ray<GBD_STORE_BF16_F16U, DEPTH, true, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
+            march_ray<GBD_STORE_BF16_F16U, DEPTH, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
                                                               R.samples, a.error_word, s_tab);
         else
-            march_ray<GBD_STORE_BF16_F16U, DEPTH, false, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
+            march_ray<GBD_STORE_BF16_F16U, DEPTH, false>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
                                                                R.samples, a.error_word, s_tab);
     }
 }
 
 // Region schedule (RegionArgs): CTA (x, y) marches rays of one view through
-// region y.  The region's table terms along each axis (forward or reversed,
-// as the view needs), followed by two sentinels, are staged in shared memory.
+// region y.  The region's table entries along each axis (forward or reversed,
+// as the view needs) are staged in shared memory.
 // The view's pixels whose rays can cross the region lie in the projection of
 // the region's box; the CTA takes one packet of that rectangle per warp,
 // keeps the rays that cross the box, sorts them by the length of their chord
@@ -1657,7 +1408,7 @@ __device__ __forceinline__ RegionFrame region_frame(const RegionArgs &a, int vi,
         const bool mirrored = (V.flags & (kFlagMirror0 << i)) != 0u;
         F.B.lo[i] = mirrored ? n - ohi : olo;
         F.B.hi[i] = mirrored ? n - olo : ohi;
-        F.B.cur0[i] = 4u * static_cast<uint32_t>(i * (a.region + 2));
+        F.B.cur0[i] = 4u * static_cast<uint32_t>(i * (a.region + 1));
         F.slot += mirrored ? a.nreg[i] - 1 - rr[i] : rr[i];
         const float c = 0.5f * static_cast<float>(F.B.lo[i] + F.B.hi[i]);
         const float h = 0.5f * static_cast<float>(F.B.hi[i] - F.B.lo[i]);
@@ -1849,11 +1600,9 @@ __global__ void __launch_bounds__(256, MINB) region_kernel(const __grid_constant
     for (int i = 0; i < 3; ++i) {
         const bool mirrored = (V.flags & (kFlagMirror0 << i)) != 0u;
         const int len = F.B.hi[i] - F.B.lo[i];
-        const int src = march_table_base(a.vol.n, i) + (mirrored ? a.vol.n[i] + 2 : 0) + F.B.lo[i];
-        for (int j = threadIdx.x; j < len + 2; j += blockDim.x)
-            s_tab[i * (a.region + 2) + j] = j < len ? a.vol.mtab[src + j] : kTabSentinel;
+        const int src = march_table_base(a.vol.n, i) + (mirrored ? a.vol.n[i] + 1 : 0) + F.B.lo[i];
+        for (int j = threadIdx.x; j < len + 1; j += blockDim.x) s_tab[i * (a.region + 1) + j] = a.vol.mtab[src + j];
     }
-    if (threadIdx.x < kTabPad) s_tab[3 * (a.region + 2) + threadIdx.x] = kTabSentinel;
     const int k = first + warp * 32 + lane;
     const uint32_t *list = a.rays + (static_cast<long long>(r) * a.n_views + vi) * a.ctas_per_view * a.rays_per_cta;
     const uint32_t pq = k < count ? __ldg(list + k) : (static_cast<uint32_t>(a.width) | (static_cast<uint32_t>(a.height) << 16));
@@ -1861,7 +1610,7 @@ __global__ void __launch_bounds__(256, MINB) region_kernel(const __grid_constant
     if (__all_sync(kFull, k >= count)) return;
     float *out = a.partial + static_cast<long long>(F.slot) * a.slot_stride +
                  static_cast<long long>(a.image[vi]) * a.width * a.height;
-    march_ray<STORE, DEPTH, PAIRED, true, true>(a.vol, V, F.B, static_cast<int>(pq & 0xffffu), static_cast<int>(pq >> 16),
+    march_ray<STORE, DEPTH, PAIRED, true>(a.vol, V, F.B, static_cast<int>(pq & 0xffffu), static_cast<int>(pq >> 16),
                                                 a.width, a.height, out, nullptr, a.error_word, s_tab);
 }
 
@@ -1909,40 +1658,34 @@ void *select_cap(int depth, int capped, bool steal)
     return capped ? select_depth<STORE, 3, PAIRED>(depth, steal) : select_depth<STORE, 1, PAIRED>(depth, steal);
 }
 
-template <int STORE, bool PAIRED, int DEPTH>
-void *select_group_depth(int size)
+template <int STORE, int DEPTH, int G>
+void *select_group_snaps(int snaps)
 {
-    if (size == 4) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, PAIRED, 4>);
-    if (size == kGroupMax) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, PAIRED, kGroupMax>);
+    if (snaps == kGroupSnapsMin) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, G, kGroupSnapsMin>);
+    if (snaps == kGroupSnapsMax) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, G, kGroupSnapsMax>);
     return nullptr;
 }
 
-template <int STORE, bool PAIRED>
-void *select_group_size(int size, int depth)
+template <int STORE, int DEPTH>
+void *select_group_size(int size, int snaps)
 {
-    // float32 groups march one cell per iteration whatever the depth: with two
-    // or four, the extra record registers cost more warps than the loads gain
-    if constexpr (STORE == GBD_STORE_F32) {
-        return (depth == 1 || depth == 2 || depth == 4) ? select_group_depth<STORE, PAIRED, 1>(size) : nullptr;
-    } else {
-        switch (depth) {
-        case 1: return select_group_depth<STORE, PAIRED, 1>(size);
-        case 2: return select_group_depth<STORE, PAIRED, 2>(size);
-        case 4: return select_group_depth<STORE, PAIRED, 4>(size);
-        default: return nullptr;
-        }
-    }
+    return size == 4 ? select_group_snaps<STORE, DEPTH, 4>(snaps)
+                     : (size == kGroupMax ? select_group_snaps<STORE, DEPTH, kGroupMax>(snaps) : nullptr);
 }
 
-// Time groups: a kernel for groups of up to 4 views and one for up to 8.
-void *select_group(int store, int paired, int size, int depth)
+// Time groups: a kernel for groups of up to 4 views and one for up to 8, each
+// for members within one snapshot of each other and within kGroupSnapsMax - 2.
+// float32 groups march one cell per iteration whatever the depth, and
+// bfloat16/float16 ones at most two: a cell's S gathers already keep as many
+// loads in flight, and more cells' records would cost more warps than the
+// loads gain.
+void *select_group(int store, int size, int depth, int snaps)
 {
-    if (store == GBD_STORE_F32)
-        return paired ? select_group_size<GBD_STORE_F32, true>(size, depth)
-                      : select_group_size<GBD_STORE_F32, false>(size, depth);
+    if (depth != 1 && depth != 2 && depth != 4) return nullptr;
+    if (store == GBD_STORE_F32) return select_group_size<GBD_STORE_F32, 1>(size, snaps);
     if (store == GBD_STORE_BF16_F16U)
-        return paired ? select_group_size<GBD_STORE_BF16_F16U, true>(size, depth)
-                      : select_group_size<GBD_STORE_BF16_F16U, false>(size, depth);
+        return depth == 1 ? select_group_size<GBD_STORE_BF16_F16U, 1>(size, snaps)
+                          : select_group_size<GBD_STORE_BF16_F16U, 2>(size, snaps);
     return nullptr;
 }
 
@@ -2017,7 +1760,7 @@ cudaError_t launch_wave(const WaveArgs &a, const LaunchCfg &cfg, cudaStream_t st
     // shared memory for the largest march tables of the launch
     int smem = 0;
     for (int r = 0; r < a.n_reqs; ++r)
-        smem = std::max(smem, static_cast<int>(sizeof(int32_t)) * (march_table_entries(a.reqs[r].vol.n) + kTabPad));
+        smem = std::max(smem, static_cast<int>(sizeof(int32_t)) * march_table_entries(a.reqs[r].vol.n));
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
@@ -2091,7 +1834,7 @@ cudaError_t launch_region(const RegionArgs &a, const LaunchCfg &cfg, cudaStream_
     if (!k || a.n_views < 1 || a.n_views > 65535 || regions < 1 || regions > 65535 || a.ctas_per_view < 1 ||
         a.rays_per_cta != 32 * cfg.cta_warps || !a.image || !a.region_order)
         return cudaErrorInvalidValue;
-    const int smem = static_cast<int>(sizeof(int32_t)) * (3 * (a.region + 2) + kTabPad);
+    const int smem = static_cast<int>(sizeof(int32_t)) * 3 * (a.region + 1);
     void *params[] = {const_cast<RegionArgs *>(&a)};
     return cudaLaunchKernel(k, dim3(static_cast<unsigned>(a.ctas_per_view), static_cast<unsigned>(a.n_views),
                                     static_cast<unsigned>(regions)),
@@ -2114,7 +1857,7 @@ cudaError_t plan_march(MarchArgs &a, const LaunchCfg &cfg, int num_sms, const do
 {
     // n_groups > 0: time groups, one unit of CTAs per group; else one per view
     const bool grouped = a.n_groups > 0;
-    void *k = grouped ? select_group(a.vol.store, a.vol.paired, a.group_size, cfg.depth)
+    void *k = grouped ? select_group(a.vol.store, a.group_size, cfg.depth, a.group_snaps)
                       : select_kernel(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired,
                                       a.persistent && a.n_views > 1);
     if (!k || a.n_views < 1 || a.n_views > kViewsPerLaunch) return cudaErrorInvalidValue;
@@ -2130,7 +1873,7 @@ cudaError_t plan_march(MarchArgs &a, const LaunchCfg &cfg, int num_sms, const do
         for (int v = v0; v < v1; ++v) uwork[u] += work ? std::max(work[v], 0.0) : 1.0;
     }
     const int threads = 32 * cfg.cta_warps;
-    const int smem = static_cast<int>(sizeof(int32_t)) * (march_table_entries(a.vol.n) + kTabPad);
+    const int smem = static_cast<int>(sizeof(int32_t)) * march_table_entries(a.vol.n);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
