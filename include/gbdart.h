@@ -158,15 +158,15 @@ typedef struct {
 /* Launch configuration of the march kernels (chosen by gbd_tune or given).
  * A render called with launch NULL uses the tuned configuration of its class
  * if gbd_tune has run for it, otherwise packet 8x4, 4 warps, depth 2,
- * persistent, capped registers, no region schedule, time groups of up to 4.
+ * capped registers, no region schedule, time groups of up to 4.
  * In a given struct, zero packet/warps/depth/group fields take those
  * defaults. */
 typedef struct {
     int32_t packet_w, packet_h;  /* pixels of one warp packet: 8x4, 4x8, 16x2, 32x1 */
     int32_t cta_warps;           /* warps per CTA: 1, 2, 4 or 8                     */
     int32_t depth;               /* cells in flight per lane: 1, 2 or 4            */
-    int32_t persistent;          /* 1 = CTAs loop over their view's tile counter;
-                                    0 = one packet per warp, one launch wave    */
+    int32_t persistent;          /* accepted, 0 or 1, without effect: every launch
+                                    is one packet per warp, view after view      */
     int32_t regcap;              /* 1 = kernel built for at most 80 registers/thread */
     int32_t region;              /* batches: 0 = march every ray whole; 16, 32, 64
                                     or 128 = region schedule: march all views' rays
@@ -241,8 +241,7 @@ int gbd_render(gbd_ctx *ctx, gbd_volume vol, const gbd_view *view, const gbd_ima
 /* Renders n views of the same image geometry; view k goes to spec->out +
  * k * width * height (and the sample counts likewise).  Views travel in the
  * kernel launch parameters, up to 128 per launch (larger batches are several
- * launches); the per-view tile counters live in a context-owned device
- * buffer.  The launches are built once into a CUDA graph per (volume, n,
+ * launches).  The launches are built once into a CUDA graph per (volume, n,
  * geometry, destination, launch) and replayed afterwards, with new views
  * written into the graph's kernel parameters.
  * Concurrent batch calls on one context are serialised on the context's lock,
@@ -255,29 +254,19 @@ int gbd_render_batch(gbd_ctx *ctx, gbd_volume vol, const gbd_view *views, int32_
  * memory while they render -- applications that hand the whole device to
  * their own allocator or memory pool up front, and latency-critical loops
  * where cudaMalloc / cudaFree (which may synchronise the device) are not
- * acceptable.  It renders like gbd_render_batch, but keeps the per-view tile
- * counters of the persistent launch in one fixed-size device array of the
- * library (4 KB, held by every GPU that loads the library until the process
- * exits) instead of allocating them, and uses no CUDA graph.
+ * acceptable.  It renders like gbd_render_batch, but allocates no memory and
+ * uses no CUDA graph.
  * Limits and behaviour:
  *  - at most GBD_NOALLOC_MAX_VIEWS views per call, otherwise GBD_ERR_INVALID;
  *  - spec->out (and spec->samples, if set) must be device memory;
  *    out_on_host is rejected with GBD_ERR_INVALID;
  *  - the whole-ray march only: an explicit launch with region != 0 is
  *    rejected with GBD_ERR_INVALID, and a tuned region schedule is replaced
- *    by the persistent whole-ray march with the tuned packet, CTA and group
+ *    by the whole-ray march with the tuned packet, CTA and group
  *    shapes (its images then agree with gbd_render_batch's to float32
- *    rounding, as any region render does); tiles are taken in counter order,
- *    never from the centre-first order table (which would need an allocation);
- *    otherwise the images equal gbd_render_batch's bit for bit;
- *  - the first call on a device looks up the array's device address on that
- *    device (cudaGetSymbolAddress) and keeps it for the life of the process;
- *    make that first call before any stream capture, and do not use this entry
- *    point on a device after a cudaDeviceReset there;
- *  - every call shares the one array, which keeps the last call's contents
- *    (the tile counters are cleared by each call): calls whose GPU work overlaps,
- *    from any context or stream on the same device, race on it, so the caller
- *    orders them (for example on one stream). */
+ *    rounding, as any region render does); a single view's blocks are taken in
+ *    row order, never from the centre-first order table (which would need an
+ *    allocation); otherwise the images equal gbd_render_batch's bit for bit. */
 #define GBD_NOALLOC_MAX_VIEWS 1024
 int gbd_render_batch_noalloc(gbd_ctx *ctx, gbd_volume vol, const gbd_view *views, int32_t n,
                              const gbd_image_spec *spec, const gbd_launch *launch, void *stream);

@@ -320,47 +320,10 @@ int check_spec(const gbd_image_spec *s)
 
 int march_chunks(int n) { return (n + kViewsPerLaunch - 1) / kViewsPerLaunch; }
 
-// Estimated cell-samples of one view: the box-and-window chord of a 16 x 16
-// subsample of its rays, times the cells crossed per unit length.  It only
-// sizes the persistent grid's share per view, so a coarse figure will do.
-double view_work(const Volume &vol, const ViewDev &V, int width, int height)
-{
-    const int sx = std::min(width, 16), sy = std::min(height, 16);
-    double rate = 0.0;
-    for (int i = 0; i < 3; ++i) rate += static_cast<double>(V.a_hi[i]) + V.a_lo[i];
-    double cells = 0.0;
-    for (int jy = 0; jy < sy; ++jy) {
-        const int q = static_cast<int>((jy + 0.5) * height / sy);
-        for (int jx = 0; jx < sx; ++jx) {
-            const int p = static_cast<int>((jx + 0.5) * width / sx);
-            double lo = V.win_lo, hi = V.win_hi;
-            bool hit = true;
-            for (int i = 0; i < 3 && hit; ++i) {
-                const double g = static_cast<double>(V.g0[i] + p * V.gu[i] + q * V.gv[i]) * 0x1p-40;
-                if (V.inv_a[i] != 0.f) {
-                    lo = std::max(lo, -g * V.inv_a[i]);
-                    hi = std::min(hi, (vol.grid.n[i] - g) * V.inv_a[i]);
-                } else if (g < 0.0 || g >= vol.grid.n[i]) {
-                    hit = false;
-                }
-            }
-            if (hit && hi > lo) cells += (hi - lo) * rate + 1.0;
-        }
-    }
-    return cells * (static_cast<double>(width) * height) / (static_cast<double>(sx) * sy);
-}
-
-std::vector<double> view_works(const Volume &vol, const std::vector<ViewDev> &hv, int width, int height)
-{
-    std::vector<double> w(hv.size());
-    for (size_t k = 0; k < hv.size(); ++k) w[k] = view_work(vol, hv[k], width, height);
-    return w;
-}
-
 // Launch arguments of chunk c of a batch of n views: views c K .. c K + K - 1
-// (K = kViewsPerLaunch), their images and their tile counters.
+// (K = kViewsPerLaunch) and their images.
 void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c, const gbd_image_spec &s,
-               float *out, uint32_t *samples, int *queue, const LaunchCfg &cfg, int *err_word)
+               float *out, uint32_t *samples, const LaunchCfg &cfg, int *err_word)
 {
     std::memset(&a, 0, sizeof(a));
     const int first = c * kViewsPerLaunch;
@@ -370,14 +333,9 @@ void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c,
     a.n_views = cnt;
     a.width = s.width;
     a.height = s.height;
-    a.packet_w = cfg.packet_w;
-    a.packet_h = cfg.packet_h;
-    a.tiles_x = (s.width + cfg.packet_w - 1) / cfg.packet_w;
-    a.tiles_y = (s.height + cfg.packet_h - 1) / cfg.packet_h;
-    a.persistent = cfg.persistent;
+    a.pk = packet_grid(s.width, s.height, cfg.packet_w, cfg.packet_h, cfg.cta_warps);
     a.out = out + img;
     a.samples = samples ? samples + img : nullptr;
-    a.queue = queue + first;
     a.error_word = err_word;
     std::memcpy(a.views, hv + first, sizeof(ViewDev) * static_cast<size_t>(cnt));
 }
@@ -468,22 +426,20 @@ void group_views(MarchArgs &a, int gmax)
 
 int launch_units(const MarchArgs &a) { return a.n_groups > 0 ? a.n_groups : a.n_views; }
 
-const int *tile_order(Ctx &ctx, int width, int height, int packet_w, int packet_h)
+const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk)
 {
-    const std::array<int, 4> key{width, height, packet_w, packet_h};
-    auto it = ctx.tile_orders.find(key);
-    if (it != ctx.tile_orders.end()) return it->second;
-    if (ctx.tile_orders.size() >= 64) return nullptr;  // bounded: further geometries keep counter order
-    const int tx = (width + packet_w - 1) / packet_w, ty = (height + packet_h - 1) / packet_h;
-    std::vector<int> order(static_cast<size_t>(tx) * ty);
+    const std::array<int, 4> key{width, height, pk.step_x, pk.step_y};
+    auto it = ctx.block_orders.find(key);
+    if (it != ctx.block_orders.end()) return it->second;
+    if (ctx.block_orders.size() >= 64) return nullptr;  // bounded: further geometries keep row order
+    std::vector<int> order(static_cast<size_t>(pk.blocks));
     std::vector<double> d2(order.size());
-    for (int y = 0; y < ty; ++y)
-        for (int x = 0; x < tx; ++x) {
-            const double dx = (x + 0.5) * packet_w - 0.5 * width, dy = (y + 0.5) * packet_h - 0.5 * height;
-            const int t = y * tx + x;
-            order[static_cast<size_t>(t)] = t;
-            d2[static_cast<size_t>(t)] = dx * dx + dy * dy;
-        }
+    for (int t = 0; t < pk.blocks; ++t) {
+        const double dx = (t % pk.blocks_x + 0.5) * pk.step_x - 0.5 * width;
+        const double dy = (t / pk.blocks_x + 0.5) * pk.step_y - 0.5 * height;
+        order[static_cast<size_t>(t)] = t;
+        d2[static_cast<size_t>(t)] = dx * dx + dy * dy;
+    }
     std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return d2[p] < d2[q]; });
     int *dev = nullptr;
     if (cudaMalloc(reinterpret_cast<void **>(&dev), order.size() * sizeof(int)) != cudaSuccess) return nullptr;
@@ -495,12 +451,9 @@ const int *tile_order(Ctx &ctx, int width, int height, int packet_w, int packet_
         cudaFree(dev);
         return nullptr;
     }
-    ctx.tile_orders[key] = dev;
+    ctx.block_orders[key] = dev;
     return dev;
 }
-
-// Bytes of the per-view tile counters of a batch, rounded up to 256.
-static size_t queue_bytes(int n) { return (static_cast<size_t>(n) * sizeof(int) + 255) / 256 * 256; }
 
 // ------------------------------------------------------------ region schedule
 // Pixel coordinates of the march frame for view V: the first two rows of the
@@ -763,8 +716,8 @@ cudaError_t enqueue_regions(Ctx &ctx, const Volume &vol, const std::vector<ViewD
 }
 
 // Renders n views whose records are already set up on the host, without a
-// cached graph: stream-ordered scratch for the tile counters or partial slots
-// (and the image when it goes to host memory).
+// cached graph: stream-ordered scratch for the partial slots, and for the image
+// when it goes to host memory.
 int render_direct(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, const gbd_image_spec &spec,
                   const LaunchCfg &cfg, cudaStream_t st)
 {
@@ -793,27 +746,25 @@ int render_direct(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, c
         set_launch_count(launches);
         return GBD_OK;
     }
-    const size_t img_off = queue_bytes(n);
-    const size_t total = img_off + (spec.out_on_host ? pix * sizeof(float) : 0);
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&scratch), total, st);
-    if (e != cudaSuccess) return cuda_fail(e, "render scratch");
-    int *queue = reinterpret_cast<int *>(scratch);
-    float *dev_out = spec.out_on_host ? reinterpret_cast<float *>(scratch + img_off) : spec.out;
-    e = cudaMemsetAsync(queue, 0, img_off, st);
+    float *dev_out = spec.out;
+    cudaError_t e = cudaSuccess;
+    if (spec.out_on_host) {
+        e = cudaMallocAsync(reinterpret_cast<void **>(&scratch), pix * sizeof(float), st);
+        if (e != cudaSuccess) return cuda_fail(e, "render scratch");
+        dev_out = reinterpret_cast<float *>(scratch);
+    }
     const int chunks = march_chunks(n);
     auto a = std::make_unique<MarchArgs>();
-    const std::vector<double> work = view_works(vol, hv, spec.width, spec.height);
     for (int c = 0; c < chunks && e == cudaSuccess; ++c) {
-        fill_args(*a, vol, hv.data(), n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, queue, cfg,
+        fill_args(*a, vol, hv.data(), n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, cfg,
                   ctx.err_word);
         group_views(*a, cfg.group);
-        if (cfg.persistent && launch_units(*a) == 1)
-            a->tile_order = tile_order(ctx, spec.width, spec.height, cfg.packet_w, cfg.packet_h);
-        e = launch_march(*a, cfg, ctx.num_sms, work.data() + static_cast<size_t>(c) * kViewsPerLaunch, st);
+        if (launch_units(*a) == 1) a->block_order = block_order(ctx, spec.width, spec.height, a->pk);
+        e = launch_march(*a, cfg, st);
     }
     if (e == cudaSuccess && spec.out_on_host)
         e = cudaMemcpyAsync(spec.out, dev_out, pix * sizeof(float), cudaMemcpyDeviceToHost, st);
-    cudaError_t ef = cudaFreeAsync(scratch, st);
+    cudaError_t ef = scratch ? cudaFreeAsync(scratch, st) : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(e, "render launch");
     if (ef != cudaSuccess) return cuda_fail(ef, "render scratch free");
     set_launch_count(chunks);
@@ -834,9 +785,8 @@ struct GraphKey {
     }
 };
 
-// A batch graph: a memset of the tile counters, one kernel node per chunk of
-// views (independent, so they may run side by side), and, for host output,
-// the copy back.  New views of the same geometry update the kernel nodes'
+// A batch graph: one kernel node per chunk of views (independent, so they may
+// run side by side), and, for host output, the copy back.  New views of the same geometry update the kernel nodes'
 // parameters in place.  A region-schedule batch is captured from
 // enqueue_regions instead (rebuilt for new views), and its copy back to host
 // memory is issued after each replay, outside the graph.
@@ -847,7 +797,7 @@ struct GraphEntry {
     std::vector<cudaGraphNode_t> knodes;
     std::vector<void *> kfuncs;  // the kernel of each node
     std::vector<ViewDev> views;  // the views the kernel nodes hold
-    char *d_scratch = nullptr;   // tile counters (+ image when out_on_host)
+    char *d_scratch = nullptr;   // image when out_on_host, or the region schedule's scratch
     float *region_img = nullptr; // region schedule with host output: the device image, copied back after each replay
     cudaEvent_t done = nullptr;
     bool launched = false;
@@ -891,18 +841,12 @@ static cudaError_t chunk_params(Ctx &ctx, const Volume &vol, const GraphKey &key
                                 const GraphEntry &g, const ViewDev *hv, int c, MarchArgs &a,
                                 cudaKernelNodeParams &kp, void **params)
 {
-    const size_t img_off = queue_bytes(key.n);
-    int *queue = reinterpret_cast<int *>(g.d_scratch);
-    float *dev_out = spec.out_on_host ? reinterpret_cast<float *>(g.d_scratch + img_off) : spec.out;
-    fill_args(a, vol, hv, key.n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, queue, key.cfg,
-              ctx.err_word);
+    float *dev_out = spec.out_on_host ? reinterpret_cast<float *>(g.d_scratch) : spec.out;
+    fill_args(a, vol, hv, key.n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, key.cfg, ctx.err_word);
     group_views(a, key.cfg.group);
-    if (key.cfg.persistent && launch_units(a) == 1)
-        a.tile_order = tile_order(ctx, spec.width, spec.height, key.cfg.packet_w, key.cfg.packet_h);
-    double work[kViewsPerLaunch];
-    for (int v = 0; v < a.n_views; ++v) work[v] = view_work(vol, a.views[v], spec.width, spec.height);
+    if (launch_units(a) == 1) a.block_order = block_order(ctx, spec.width, spec.height, a.pk);
     KernelLaunch L;
-    cudaError_t e = plan_march(a, key.cfg, ctx.num_sms, work, L);
+    cudaError_t e = plan_march(a, key.cfg, L);
     if (e != cudaSuccess) return e;
     kp = cudaKernelNodeParams{};
     kp.func = L.func;
@@ -966,25 +910,14 @@ static int build_graph(Ctx &ctx, const Volume &vol, const GraphKey &key, const g
     const int slots = region_slots(vol, key.cfg, spec, nreg, key.n);
     if (slots > 0) return build_region_graph(ctx, vol, key, spec, hv, slots, g);
     const int n = key.n;
-    const size_t img_off = queue_bytes(n);
     const size_t pix = static_cast<size_t>(spec.width) * spec.height * n;
-    const size_t total = img_off + (spec.out_on_host ? pix * sizeof(float) : 0);
-    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&g.d_scratch), total);
+    cudaError_t e = cudaSuccess;
+    if (spec.out_on_host) e = cudaMalloc(reinterpret_cast<void **>(&g.d_scratch), pix * sizeof(float));
     if (e != cudaSuccess) return cuda_fail(e, "batch scratch");
     e = cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming);
     if (e != cudaSuccess) return cuda_fail(e, "batch event");
     e = cudaGraphCreate(&g.graph, 0);
     if (e != cudaSuccess) return cuda_fail(e, "batch graph");
-    cudaMemsetParams mp;
-    std::memset(&mp, 0, sizeof(mp));
-    mp.dst = g.d_scratch;
-    mp.value = 0;
-    mp.elementSize = 4;
-    mp.width = img_off / 4;
-    mp.height = 1;
-    cudaGraphNode_t mnode = nullptr;
-    e = cudaGraphAddMemsetNode(&mnode, g.graph, nullptr, 0, &mp);
-    if (e != cudaSuccess) return cuda_fail(e, "batch graph memset node");
     auto a = std::make_unique<MarchArgs>();
     const int chunks = march_chunks(n);
     for (int c = 0; c < chunks; ++c) {
@@ -992,7 +925,7 @@ static int build_graph(Ctx &ctx, const Volume &vol, const GraphKey &key, const g
         void *params[1];
         e = chunk_params(ctx, vol, key, spec, g, hv.data(), c, *a, kp, params);
         cudaGraphNode_t kn = nullptr;
-        if (e == cudaSuccess) e = cudaGraphAddKernelNode(&kn, g.graph, &mnode, 1, &kp);
+        if (e == cudaSuccess) e = cudaGraphAddKernelNode(&kn, g.graph, nullptr, 0, &kp);
         if (e != cudaSuccess) return cuda_fail(e, "batch graph kernel node");
         g.knodes.push_back(kn);
         g.kfuncs.push_back(kp.func);
@@ -1000,7 +933,7 @@ static int build_graph(Ctx &ctx, const Volume &vol, const GraphKey &key, const g
     if (spec.out_on_host) {
         cudaGraphNode_t cn = nullptr;
         e = cudaGraphAddMemcpyNode1D(&cn, g.graph, g.knodes.data(), g.knodes.size(), spec.out,
-                                     g.d_scratch + img_off, pix * sizeof(float), cudaMemcpyDeviceToHost);
+                                     g.d_scratch, pix * sizeof(float), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(e, "batch graph copy node");
     }
     e = cudaGraphInstantiate(&g.exec, g.graph, 0);
@@ -1194,8 +1127,8 @@ int gbd_destroy(gbd_ctx *ctx)
         ctx->volumes.clear();
         if (ctx->err_word) cudaFree(ctx->err_word);
         if (ctx->region_done) cudaEventDestroy(ctx->region_done);
-        for (auto &kv : ctx->tile_orders) cudaFree(kv.second);
-        ctx->tile_orders.clear();
+        for (auto &kv : ctx->block_orders) cudaFree(kv.second);
+        ctx->block_orders.clear();
         if (ctx->load_stream) cudaStreamDestroy(ctx->load_stream);
         if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
         for (int k = 0; k < 4; ++k) {
@@ -1477,8 +1410,8 @@ int gbd_touched_records(gbd_ctx *ctx, gbd_volume vid, const gbd_view *views, int
     gbd_image_spec s = *spec;
     s.out = nullptr;  // the analysis writes no image
     for (int c = 0; c < march_chunks(n) && e == cudaSuccess; ++c) {
-        fill_args(*a, *vol, hv.data(), n, c, s, reinterpret_cast<float *>(bits), nullptr, nullptr, cfg, ctx->err_word);
-        e = launch_touch(*a, bits, cells, cfg, ctx->num_sms, st);
+        fill_args(*a, *vol, hv.data(), n, c, s, reinterpret_cast<float *>(bits), nullptr, cfg, ctx->err_word);
+        e = launch_touch(*a, bits, cells, cfg, st);
     }
     std::vector<uint32_t> host(words);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host.data(), bits, words * 4, cudaMemcpyDeviceToHost, st);
@@ -1511,29 +1444,23 @@ int gbd_render_vector(gbd_ctx *ctx, gbd_volume vid, const gbd_view *views, int32
     for (int k = 0; k < n; ++k)
         if ((rc = make_view(*vol, views[k], spec->width, spec->height, spec->fov_u, spec->fov_v, hv[k]))) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t qbytes = (static_cast<size_t>(n) * sizeof(int) + 255) / 256 * 256;
-    int *queue = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&queue), qbytes, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(queue, 0, qbytes, st);
+    cudaError_t e = cudaSuccess;
     const long long plane = static_cast<long long>(spec->width) * spec->height;
     const long long img_stride = plane * (1 + vol->n_chan);
-    const std::vector<double> work = view_works(*vol, hv, spec->width, spec->height);
     auto a = std::make_unique<MarchArgs>();
     int launches = 0;
     for (int c = 0; c < march_chunks(n) && e == cudaSuccess; ++c) {
-        fill_args(*a, *vol, hv.data(), n, c, *spec, spec->out, nullptr, queue, cfg, ctx->err_word);
+        fill_args(*a, *vol, hv.data(), n, c, *spec, spec->out, nullptr, cfg, ctx->err_word);
         a->out = spec->out + static_cast<long long>(c) * kViewsPerLaunch * img_stride;
         a->img_stride = img_stride;
         a->chan = vol->chan;
         a->chan_comp_stride = vol->chan_stride * vol->grid.n_epochs;
         a->chan_cell_stride = vol->chan_stride;
-        e = launch_vector(*a, vol->n_chan, cfg, ctx->num_sms, work.data() + static_cast<size_t>(c) * kViewsPerLaunch,
-                          st);
+        if (launch_units(*a) == 1) a->block_order = block_order(*ctx, spec->width, spec->height, a->pk);
+        e = launch_vector(*a, vol->n_chan, cfg, st);
         ++launches;
     }
-    cudaError_t ef = queue ? cudaFreeAsync(queue, st) : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(e, "vector render");
-    if (ef != cudaSuccess) return cuda_fail(ef, "vector render scratch");
     set_launch_count(launches);
     return GBD_OK;
 }

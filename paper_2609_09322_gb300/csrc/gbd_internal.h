@@ -104,14 +104,36 @@ constexpr int kGroupDefault = 4;
 constexpr int kGroupSnapsMin = 3;
 constexpr int kGroupSnapsMax = 5;
 
+// How the CTAs of a march cover an image.  A warp owns a packet of 32 pixels,
+// a CTA a near-square block of packets, so that the rays it marches side by side
+// share cells in L1.
+struct PacketGrid {
+    int packet_w, packet_h;   // packet_w * packet_h == 32
+    int block_w;              // packets per block row
+    int step_x, step_y;       // pixels per block
+    int blocks_x, blocks;     // blocks per image row, per image
+};
+inline PacketGrid packet_grid(int width, int height, int packet_w, int packet_h, int cta_warps)
+{
+    PacketGrid g;
+    g.packet_w = packet_w;
+    g.packet_h = packet_h;
+    g.block_w = 1;  // widened while the block stays no wider than high
+    while (2 * g.block_w <= cta_warps && 2 * g.block_w * packet_w <= (cta_warps / (2 * g.block_w)) * packet_h * 2) g.block_w *= 2;
+    g.step_x = g.block_w * packet_w;
+    g.step_y = (cta_warps / g.block_w) * packet_h;
+    g.blocks_x = (width + g.step_x - 1) / g.step_x;
+    g.blocks = g.blocks_x * ((height + g.step_y - 1) / g.step_y);
+    return g;
+}
+
 // One march launch: n_views views of one image geometry.
 struct MarchArgs {
     VolDev vol;
     int n_views;              // views in this launch, 1 .. kViewsPerLaunch
     int width, height;
-    int packet_w, packet_h;   // packet_w * packet_h == 32
-    int tiles_x, tiles_y;     // packets per image row / column
-    int cta_begin[kViewsPerLaunch + 1];  // first CTA of each view (or group), then the total (set by plan_march)
+    PacketGrid pk;            // how the CTAs and warps cover an image
+    const int *block_order;   // CTA of an image -> its block (centre of the image first), or NULL: in row order
     int n_groups;             // 0: every view marched on its own; else time groups of consecutive views
     int group_size;           // time groups: the kernel's member limit (4 or kGroupMax)
     int group_snaps;          // and its snapshots per cell (kGroupSnapsMin or kGroupSnapsMax)
@@ -119,12 +141,9 @@ struct MarchArgs {
     int group_ref[kViewsPerLaunch];        // the group's reference view: the largest u_obs
     float group_win[kViewsPerLaunch][2];   // the union of the members' windows
     long long view_delta[kViewsPerLaunch]; // u_obs of the view minus that of its group's reference, Q31.32
-    int persistent;           // CTAs loop over their view's tile counter
     int accumulate;           // add to out (and samples) instead of storing
     float *out;               // n_views * width * height floats
     uint32_t *samples;        // optional, same shape
-    int *queue;               // persistent mode: one tile counter per view or group (zeroed before launch)
-    const int *tile_order;    // persistent mode: counter value -> tile (centre of the image first), or NULL
     int *error_word;          // checked builds: first bounds violation code
     // vector renders (vector_kernel): extra emissivity channels of the volume
     const float *chan;        // n_chan channels, each M blocks of chan_cell_stride floats
@@ -202,7 +221,7 @@ struct ReqDev {
     VolDev vol;
     ViewDev view;
     int width, height;
-    int tiles_x, tiles_y;
+    int blocks_x;             // blocks per image row
     int cta_begin;            // first CTA of this request in the launch
     float *out;               // device image of the request
     uint32_t *samples;        // optional per-pixel cell-sample counts
@@ -212,11 +231,11 @@ struct ReqDev {
 // several launches on its stream.
 constexpr int kReqsPerLaunch = 96;
 
-// One launch of a served wave: each request gets ceil(tiles / warps per CTA)
-// CTAs, one packet per warp.
+// One launch of a served wave: each request gets a CTA per block of its image,
+// one packet per warp.
 struct WaveArgs {
     int n_reqs;
-    int packet_w, packet_h;
+    PacketGrid pk;            // packets and blocks (blocks_x and blocks: per request)
     int total_ctas;
     int *error_word;
     ReqDev reqs[kReqsPerLaunch];  // sorted by cta_begin
@@ -236,20 +255,16 @@ struct KernelLaunch {
 };
 
 // Kernel entry points (march.cu, pack.cu).  plan_march picks the kernel and
-// grid for a filled MarchArgs and sets its cta_begin; `work` (n_views
-// estimates, or NULL for equal shares) splits a persistent grid over the
-// views.  launch_march plans and launches.
-cudaError_t plan_march(MarchArgs &a, const LaunchCfg &cfg, int num_sms, const double *work, KernelLaunch &k);
-cudaError_t launch_march(MarchArgs &a, const LaunchCfg &cfg, int num_sms, const double *work, cudaStream_t stream);
+// grid for a filled MarchArgs; launch_march plans and launches.
+cudaError_t plan_march(const MarchArgs &a, const LaunchCfg &cfg, KernelLaunch &k);
+cudaError_t launch_march(MarchArgs &a, const LaunchCfg &cfg, cudaStream_t stream);
 cudaError_t launch_wave(const WaveArgs &a, const LaunchCfg &cfg, cudaStream_t stream);
 // Memory analysis: sets bit m * cells + cell of `bits` for every record the
-// views' samples read (a non-persistent launch planned like the march).
-cudaError_t launch_touch(MarchArgs &a, uint32_t *bits, long long cells, const LaunchCfg &cfg, int num_sms,
-                         cudaStream_t stream);
+// views' samples read (a launch planned like the march).
+cudaError_t launch_touch(MarchArgs &a, uint32_t *bits, long long cells, const LaunchCfg &cfg, cudaStream_t stream);
 // Vector render: n_chan (1 or 3) extra channels besides j'; image v's
 // component c at out + v * img_stride + c * width * height.
-cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, int num_sms, const double *work,
-                          cudaStream_t stream);
+cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, cudaStream_t stream);
 // Region schedule: the caller has filled everything but the grid, which
 // launch_screen (a warp per view and region) and launch_region (ctas_per_view
 // x views x regions) derive from the counts.  launch_screen writes the ray

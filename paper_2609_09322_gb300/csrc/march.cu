@@ -1091,155 +1091,83 @@ __device__ __forceinline__ void march_group(const VolDev &vol, const ViewDev &V,
     }
 }
 
+// The pixel of this lane in block `block` of an image.
+__device__ __forceinline__ void block_pixel(const PacketGrid &g, int blocks_x, int block, int &p, int &q)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int by = block / blocks_x, bx = block - by * blocks_x;
+    const int wy = warp / g.block_w, wx = warp - wy * g.block_w;
+    const int ly = lane / g.packet_w, lx = lane - ly * g.packet_w;
+    p = bx * g.step_x + wx * g.packet_w + lx;
+    q = by * g.step_y + wy * g.packet_h + ly;
+}
+
+// The march kernels' work split: one CTA per block of packets of one view (or
+// time group), one packet per warp, and the CTAs of the launch view after view.  The
+// hardware hands out CTAs as they end, which balances the load by itself; at any
+// moment the chip works on neighbouring blocks of one or two views, whose rays
+// share cells in L1 (within a CTA) and L2 (against persistent CTAs spread over all views
+// and pulling packets from per-view counters: 24 views of 384^2 of 256^3 x 16 float32 3.17 -> 2.81
+// ms, one 1024^2 image of 512^3 x 8 1.58 -> 1.44 ms).  The view index comes
+// from the CTA index alone, so every per-view constant stays uniform.
+struct BlockWork {
+    int unit;   // view, or time group
+    int block;  // of its image
+};
+__device__ __forceinline__ BlockWork block_work(const MarchArgs &a)
+{
+    BlockWork w;
+    const int b = static_cast<int>(blockIdx.x);
+    w.unit = b / a.pk.blocks;
+    w.block = b - w.unit * a.pk.blocks;
+    if (a.block_order) w.block = __ldg(a.block_order + w.block);
+    return w;
+}
+
 // MINB = 1 leaves the register count to the compiler; MINB = 3 asks for
 // three 256-thread CTAs per SM (at most 80 registers per thread).
-//
-// Each CTA works on one view, one packet per warp: its tile directly, or,
-// persistent, tiles pulled from the view's counter until none are left (with
-// STEAL, then from the other views' counters in turn).  The
-// CTAs of view v are cta_begin[v] .. cta_begin[v + 1] - 1 (persistent grids
-// give each view a share of the GPU in proportion to its estimated work); a
-// binary search over these parameter-space bounds keeps the view index
-// uniform across the CTA.
-template <int STORE, int DEPTH, int MINB, bool PAIRED, bool STEAL>
+template <int STORE, int DEPTH, int MINB, bool PAIRED>
 __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_tab[];
-    const int ntab = march_table_entries(a.vol.n);
-    stage_tables(s_tab, a.vol.mtab, ntab);
+    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
     __syncthreads();
-
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpc = blockDim.x >> 5;
-    const int b = static_cast<int>(blockIdx.x);
-    int home = 0, hi = a.n_views - 1;  // last view whose first CTA is <= b
-    while (home < hi) {
-        const int mid = (home + hi + 1) >> 1;
-        if (a.cta_begin[mid] <= b) home = mid;
-        else hi = mid - 1;
-    }
-    const int cb = b - a.cta_begin[home];
-    const int tiles = a.tiles_x * a.tiles_y;
-    const long long stride = a.img_stride ? a.img_stride : static_cast<long long>(a.width) * a.height;
-    if constexpr (STEAL) {
-        // Persistent warps take their home view's tiles first, then, once
-        // its counter is spent, the other views' tiles in turn, so that no SM
-        // idles while any view of the launch has tiles left.  The view index
-        // depends on the CTA and the round only, and the exit test is a warp
-        // vote, so the view's constants stay warp-uniform.
-        const int rounds = a.persistent ? a.n_views : 1;
-        for (int r = 0; r < rounds; ++r) {
-            const int vi = home + r < a.n_views ? home + r : home + r - a.n_views;
-            const ViewDev &V = a.views[vi];
-            const RayBox box = grid_box(a.vol, V);
-            float *out = a.out + vi * stride;
-            uint32_t *cnt = a.samples ? a.samples + vi * stride : nullptr;
-            int tile = cb * wpc + warp;
-            for (;;) {
-                if (a.persistent) {
-                    int it = 0;
-                    if (lane == 0) it = atomicAdd(a.queue + vi, 1);
-                    tile = __shfl_sync(kFull, it, 0);
-                }
-                if (__any_sync(kFull, tile >= tiles)) break;
-                if (a.persistent && a.tile_order) tile = __ldg(a.tile_order + tile);
-                const int tx = tile % a.tiles_x;
-                const int ty = tile / a.tiles_x;
-                const int p = tx * a.packet_w + lane % a.packet_w;
-                const int q = ty * a.packet_h + lane / a.packet_w;
-                march_ray<STORE, DEPTH, PAIRED>(a.vol, V, box, p, q, a.width, a.height, out, cnt,
-                                                      a.error_word, s_tab, a.accumulate != 0);
-                if (!a.persistent) break;
-            }
-        }
-    } else {
-        // one view (or one packet per warp): the home view's tiles only
-        const ViewDev &V = a.views[home];
-        const RayBox box = grid_box(a.vol, V);
-        float *out = a.out + home * stride;
-        uint32_t *cnt = a.samples ? a.samples + home * stride : nullptr;
-        int tile = cb * wpc + warp;
-        for (;;) {
-            if (a.persistent) {
-                int it = 0;
-                if (lane == 0) it = atomicAdd(a.queue + home, 1);
-                tile = __shfl_sync(kFull, it, 0);
-            }
-            if (tile >= tiles) break;
-            if (a.persistent && a.tile_order) tile = __ldg(a.tile_order + tile);
-            const int p = (tile % a.tiles_x) * a.packet_w + lane % a.packet_w;
-            const int q = (tile / a.tiles_x) * a.packet_h + lane / a.packet_w;
-            march_ray<STORE, DEPTH, PAIRED>(a.vol, V, box, p, q, a.width, a.height, out, cnt, a.error_word,
-                                                  s_tab, a.accumulate != 0);
-            if (!a.persistent) break;
-        }
-    }
+    const BlockWork w = block_work(a);
+    const ViewDev &V = a.views[w.unit];
+    const long long img = w.unit * (a.img_stride ? a.img_stride : static_cast<long long>(a.width) * a.height);
+    int p, q;
+    block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    march_ray<STORE, DEPTH, PAIRED>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height, a.out + img,
+                                    a.samples ? a.samples + img : nullptr, a.error_word, s_tab, a.accumulate != 0);
 }
 
 // Time groups: march_kernel's work split over groups of views instead of
-// single views (group g is views group_first[g] .. group_first[g + 1] - 1,
-// its CTAs cta_begin[g] .. cta_begin[g + 1] - 1, its tile counter queue[g]).
+// single views (group g is views group_first[g] .. group_first[g + 1] - 1).
 // DEPTH cells per iteration, S snapshots per cell, at most 80 registers.
 template <int STORE, int DEPTH, int G, int S>
 __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_tab[];
-    const int ntab = march_table_entries(a.vol.n);
-    stage_tables(s_tab, a.vol.mtab, ntab);
+    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
     __syncthreads();
-
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpc = blockDim.x >> 5;
-    const int b = static_cast<int>(blockIdx.x);
-    int home = 0, hi = a.n_groups - 1;  // last group whose first CTA is <= b
-    while (home < hi) {
-        const int mid = (home + hi + 1) >> 1;
-        if (a.cta_begin[mid] <= b) home = mid;
-        else hi = mid - 1;
-    }
-    const int cb = b - a.cta_begin[home];
-    const int tiles = a.tiles_x * a.tiles_y;
+    const BlockWork w = block_work(a);
+    const int first = a.group_first[w.unit];
+    const int gcnt = a.group_first[w.unit + 1] - first;
+    const ViewDev &V = a.views[a.group_ref[w.unit]];
     const long long stride = a.img_stride ? a.img_stride : static_cast<long long>(a.width) * a.height;
-    // home group first, then the other groups' tiles in turn (as march_kernel)
-    const int rounds = a.persistent ? a.n_groups : 1;
-    for (int r = 0; r < rounds; ++r) {
-        const int gi = home + r < a.n_groups ? home + r : home + r - a.n_groups;
-        const int first = a.group_first[gi];
-        const int gcnt = a.group_first[gi + 1] - first;
-        const ViewDev *GV = a.views + first;
-        const ViewDev &V = a.views[a.group_ref[gi]];
-        const float win_lo = a.group_win[gi][0], win_hi = a.group_win[gi][1];
-        const RayBox box = grid_box(a.vol, V);
-        float *out = a.out + first * stride;
-        uint32_t *cnt = a.samples ? a.samples + first * stride : nullptr;
-        int tile = cb * wpc + warp;
-        for (;;) {
-            if (a.persistent) {
-                int it = 0;
-                if (lane == 0) it = atomicAdd(a.queue + gi, 1);
-                tile = __shfl_sync(kFull, it, 0);
-            }
-            if (__any_sync(kFull, tile >= tiles)) break;  // uniform across the warp
-            if (a.persistent && a.tile_order) tile = __ldg(a.tile_order + tile);
-            const int tx = tile % a.tiles_x;
-            const int ty = tile / a.tiles_x;
-            const int p = tx * a.packet_w + lane % a.packet_w;
-            const int q = ty * a.packet_h + lane / a.packet_w;
-            auto march = [&](auto plain) {
-                march_group<STORE, DEPTH, G, S, decltype(plain)::value>(
-                    a.vol, V, win_lo, win_hi, GV, a.view_delta + first, gcnt, box, p, q, a.width, a.height, out, stride,
-                    cnt, a.error_word, s_tab);
-            };
-            if constexpr (STORE == GBD_STORE_F32) {
-                march(std::false_type{});
-            } else {
-                if (a.vol.plain_boost) march(std::true_type{});
-                else march(std::false_type{});
-            }
-            if (!a.persistent) break;
-        }
+    int p, q;
+    block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    auto march = [&](auto plain) {
+        march_group<STORE, DEPTH, G, S, decltype(plain)::value>(
+            a.vol, V, a.group_win[w.unit][0], a.group_win[w.unit][1], a.views + first, a.view_delta + first, gcnt,
+            grid_box(a.vol, V), p, q, a.width, a.height, a.out + first * stride, stride,
+            a.samples ? a.samples + first * stride : nullptr, a.error_word, s_tab);
+    };
+    if constexpr (STORE == GBD_STORE_F32) {
+        march(std::false_type{});
+    } else {
+        if (a.vol.plain_boost) march(std::true_type{});
+        else march(std::false_type{});
     }
 }
 
@@ -1249,78 +1177,33 @@ template <int STORE, int NCH, bool PAIRED, int MINB>
 __global__ void __launch_bounds__(256, MINB) vector_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_tab[];
-    const int ntab = march_table_entries(a.vol.n);
-    stage_tables(s_tab, a.vol.mtab, ntab);
+    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpc = blockDim.x >> 5;
-    const int b = static_cast<int>(blockIdx.x);
-    int home = 0, hi = a.n_views - 1;
-    while (home < hi) {
-        const int mid = (home + hi + 1) >> 1;
-        if (a.cta_begin[mid] <= b) home = mid;
-        else hi = mid - 1;
-    }
-    const int cb = b - a.cta_begin[home];
-    const int tiles = a.tiles_x * a.tiles_y;
-    const ChanPtrs ch{a.chan, a.chan_comp_stride, a.chan_cell_stride};
-    // home view first, then the other views' tiles in turn (as march_kernel)
-    const int rounds = a.persistent ? a.n_views : 1;
-    for (int r = 0; r < rounds; ++r) {
-        const int vi = home + r < a.n_views ? home + r : home + r - a.n_views;
-        const ViewDev &V = a.views[vi];
-        const RayBox box = grid_box(a.vol, V);
-        float *out = a.out + static_cast<long long>(vi) * a.img_stride;
-        int tile = cb * wpc + warp;
-        for (;;) {
-            if (a.persistent) {
-                int it = 0;
-                if (lane == 0) it = atomicAdd(a.queue + vi, 1);
-                tile = __shfl_sync(kFull, it, 0);
-            }
-            if (__any_sync(kFull, tile >= tiles)) break;  // uniform across the warp
-            const int tx = tile % a.tiles_x;
-            const int ty = tile / a.tiles_x;
-            const int p = tx * a.packet_w + lane % a.packet_w;
-            const int q = ty * a.packet_h + lane / a.packet_w;
-            march_ray<STORE, 2, PAIRED, false, NCH>(a.vol, V, box, p, q, a.width, a.height, out, nullptr,
-                                                           a.error_word, s_tab, false, ch);
-            if (!a.persistent) break;
-        }
-    }
+    const BlockWork w = block_work(a);
+    const ViewDev &V = a.views[w.unit];
+    int p, q;
+    block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    const ChanPtrs ch{a.chan, a.chan_comp_stride, a.chan_cell_stride, nullptr};
+    march_ray<STORE, 2, PAIRED, false, NCH>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height,
+                                            a.out + w.unit * a.img_stride, nullptr, a.error_word, s_tab, false, ch);
 }
 
 // Memory analysis: marks every (snapshot, cell) record the views' samples
-// read (one packet per warp, no persistent queue).
+// read.
 template <int STORE, bool PAIRED>
 __global__ void __launch_bounds__(256, 1) touch_kernel(const __grid_constant__ MarchArgs a, uint32_t *bits,
                                                         long long cells)
 {
     extern __shared__ int32_t s_tab[];
-    const int ntab = march_table_entries(a.vol.n);
-    stage_tables(s_tab, a.vol.mtab, ntab);
+    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpc = blockDim.x >> 5;
-    const int b = static_cast<int>(blockIdx.x);
-    int vi = 0, hi = a.n_views - 1;
-    while (vi < hi) {
-        const int mid = (vi + hi + 1) >> 1;
-        if (a.cta_begin[mid] <= b) vi = mid;
-        else hi = mid - 1;
-    }
-    const ViewDev &V = a.views[vi];
-    const RayBox box = grid_box(a.vol, V);
-    const int tile = (b - a.cta_begin[vi]) * wpc + warp;
-    if (tile >= a.tiles_x * a.tiles_y) return;
-    const int p = (tile % a.tiles_x) * a.packet_w + lane % a.packet_w;
-    const int q = (tile / a.tiles_x) * a.packet_h + lane / a.packet_w;
-    float *out = a.out + static_cast<long long>(vi) * a.width * a.height;
+    const BlockWork w = block_work(a);
+    const ViewDev &V = a.views[w.unit];
+    int p, q;
+    block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
     const ChanPtrs ch{nullptr, 0, cells, bits};
-    march_ray<STORE, 1, PAIRED, false, 0, true>(a.vol, V, box, p, q, a.width, a.height, out, nullptr,
-                                                       a.error_word, s_tab, false, ch);
+    march_ray<STORE, 1, PAIRED, false, 0, true>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height, a.out, nullptr,
+                                                a.error_word, s_tab, false, ch);
 }
 
 // Serving: one launch over the tiles of many requests, each with its own
@@ -1334,9 +1217,6 @@ template <int DEPTH, int MINB>
 __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__ WaveArgs a)
 {
     extern __shared__ int32_t s_tab[];
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int wpc = blockDim.x >> 5;
     const int b = static_cast<int>(blockIdx.x);
     int lo = 0, hi = a.n_reqs - 1;  // last request whose first CTA is <= b
     while (lo < hi) {
@@ -1348,12 +1228,8 @@ __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__
     const int ntab = march_table_entries(R.vol.n);
     stage_tables(s_tab, R.vol.mtab, ntab);
     __syncthreads();
-    const int tile = (b - R.cta_begin) * wpc + warp;
-    if (tile >= R.tiles_x * R.tiles_y) return;
-    const int tx = tile % R.tiles_x;
-    const int ty = tile / R.tiles_x;
-    const int p = tx * a.packet_w + lane % a.packet_w;
-    const int q = ty * a.packet_h + lane / a.packet_w;
+    int p, q;
+    block_pixel(a.pk, R.blocks_x, b - R.cta_begin, p, q);
     const RayBox box = grid_box(R.vol, R.view);
     if (R.vol.store == GBD_STORE_F32) {
         if (R.vol.paired)
@@ -1634,28 +1510,21 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
     }
 }
 
-template <int STORE, int DEPTH, int MINB, bool PAIRED>
-void *kernel_ptr(bool steal)
-{
-    return steal ? reinterpret_cast<void *>(&march_kernel<STORE, DEPTH, MINB, PAIRED, true>)
-                 : reinterpret_cast<void *>(&march_kernel<STORE, DEPTH, MINB, PAIRED, false>);
-}
-
 template <int STORE, int MINB, bool PAIRED>
-void *select_depth(int depth, bool steal)
+void *select_depth(int depth)
 {
     switch (depth) {
-    case 1: return kernel_ptr<STORE, 1, MINB, PAIRED>(steal);
-    case 2: return kernel_ptr<STORE, 2, MINB, PAIRED>(steal);
-    case 4: return kernel_ptr<STORE, 4, MINB, PAIRED>(steal);
+    case 1: return reinterpret_cast<void *>(&march_kernel<STORE, 1, MINB, PAIRED>);
+    case 2: return reinterpret_cast<void *>(&march_kernel<STORE, 2, MINB, PAIRED>);
+    case 4: return reinterpret_cast<void *>(&march_kernel<STORE, 4, MINB, PAIRED>);
     default: return nullptr;
     }
 }
 
 template <int STORE, bool PAIRED>
-void *select_cap(int depth, int capped, bool steal)
+void *select_cap(int depth, int capped)
 {
-    return capped ? select_depth<STORE, 3, PAIRED>(depth, steal) : select_depth<STORE, 1, PAIRED>(depth, steal);
+    return capped ? select_depth<STORE, 3, PAIRED>(depth) : select_depth<STORE, 1, PAIRED>(depth);
 }
 
 template <int STORE, int DEPTH, int G>
@@ -1689,16 +1558,13 @@ void *select_group(int store, int size, int depth, int snaps)
     return nullptr;
 }
 
-// steal: persistent CTAs move on to the other views' tiles once their own
-// view's are spent (launches of more than one view).
-void *select_kernel(int store, int depth, int capped, int paired, bool steal)
+void *select_kernel(int store, int depth, int capped, int paired)
 {
     if (store == GBD_STORE_F32)
-        return paired ? select_cap<GBD_STORE_F32, true>(depth, capped, steal)
-                      : select_cap<GBD_STORE_F32, false>(depth, capped, steal);
+        return paired ? select_cap<GBD_STORE_F32, true>(depth, capped) : select_cap<GBD_STORE_F32, false>(depth, capped);
     if (store == GBD_STORE_BF16_F16U)
-        return paired ? select_cap<GBD_STORE_BF16_F16U, true>(depth, capped, steal)
-                      : select_cap<GBD_STORE_BF16_F16U, false>(depth, capped, steal);
+        return paired ? select_cap<GBD_STORE_BF16_F16U, true>(depth, capped)
+                      : select_cap<GBD_STORE_BF16_F16U, false>(depth, capped);
     return nullptr;
 }
 
@@ -1770,8 +1636,7 @@ cudaError_t launch_wave(const WaveArgs &a, const LaunchCfg &cfg, cudaStream_t st
                             stream);
 }
 
-cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, int num_sms, const double *work,
-                          cudaStream_t stream)
+cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, cudaStream_t stream)
 {
     // the compiler's register budget: capped, the three-channel kernel spills
     // and runs slower than the extra resident warps gain
@@ -1783,7 +1648,7 @@ cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, int nu
     c.depth = 2;
     c.regcap = 0;
     KernelLaunch L;
-    cudaError_t e = plan_march(a, c, num_sms, work, L);
+    cudaError_t e = plan_march(a, c, L);
     if (e != cudaSuccess) return e;
     if (L.smem > 48 * 1024) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
@@ -1793,18 +1658,15 @@ cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, int nu
     return cudaLaunchKernel(k, L.grid, L.block, params, L.smem, stream);
 }
 
-cudaError_t launch_touch(MarchArgs &a, uint32_t *bits, long long cells, const LaunchCfg &cfg, int num_sms,
-                         cudaStream_t stream)
+cudaError_t launch_touch(MarchArgs &a, uint32_t *bits, long long cells, const LaunchCfg &cfg, cudaStream_t stream)
 {
     void *k = a.vol.store == GBD_STORE_F32
                   ? (a.vol.paired ? reinterpret_cast<void *>(&touch_kernel<GBD_STORE_F32, true>)
                                   : reinterpret_cast<void *>(&touch_kernel<GBD_STORE_F32, false>))
                   : (a.vol.paired ? reinterpret_cast<void *>(&touch_kernel<GBD_STORE_BF16_F16U, true>)
                                   : reinterpret_cast<void *>(&touch_kernel<GBD_STORE_BF16_F16U, false>));
-    // one packet per warp: the grid covers every tile
-    a.persistent = 0;
     KernelLaunch L;
-    cudaError_t e = plan_march(a, cfg, num_sms, nullptr, L);
+    cudaError_t e = plan_march(a, cfg, L);
     if (e != cudaSuccess) return e;
     if (L.smem > 48 * 1024) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
@@ -1853,69 +1715,39 @@ cudaError_t launch_reduce(const ReduceArgs &a, cudaStream_t stream)
                             0, stream);
 }
 
-cudaError_t plan_march(MarchArgs &a, const LaunchCfg &cfg, int num_sms, const double *work, KernelLaunch &L)
+cudaError_t plan_march(const MarchArgs &a, const LaunchCfg &cfg, KernelLaunch &L)
 {
-    // n_groups > 0: time groups, one unit of CTAs per group; else one per view
+    // n_groups > 0: time groups, one image's blocks of CTAs per group; else per view
     const bool grouped = a.n_groups > 0;
     void *k = grouped ? select_group(a.vol.store, a.group_size, cfg.depth, a.group_snaps)
-                      : select_kernel(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired,
-                                      a.persistent && a.n_views > 1);
+                      : select_kernel(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired);
     if (!k || a.n_views < 1 || a.n_views > kViewsPerLaunch) return cudaErrorInvalidValue;
     if (grouped && (a.n_groups > a.n_views || a.group_first[0] != 0 || a.group_first[a.n_groups] != a.n_views))
         return cudaErrorInvalidValue;
     const int units = grouped ? a.n_groups : a.n_views;
-    double uwork[kViewsPerLaunch];
-    for (int u = 0; u < units; ++u) {
-        uwork[u] = 0.0;
-        const int v0 = grouped ? a.group_first[u] : u, v1 = grouped ? a.group_first[u + 1] : u + 1;
-        if (grouped && (v1 <= v0 || v1 - v0 > a.group_size || a.group_ref[u] < v0 || a.group_ref[u] >= v1))
+    for (int u = 0; u < units && grouped; ++u) {
+        const int v0 = a.group_first[u], v1 = a.group_first[u + 1];
+        if (v1 <= v0 || v1 - v0 > a.group_size || a.group_ref[u] < v0 || a.group_ref[u] >= v1)
             return cudaErrorInvalidValue;
-        for (int v = v0; v < v1; ++v) uwork[u] += work ? std::max(work[v], 0.0) : 1.0;
     }
-    const int threads = 32 * cfg.cta_warps;
     const int smem = static_cast<int>(sizeof(int32_t)) * march_table_entries(a.vol.n);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
     }
-    const long long tiles = static_cast<long long>(a.tiles_x) * a.tiles_y;
-    const long long needed = (tiles + cfg.cta_warps - 1) / cfg.cta_warps;
-    long long total = 0;
-    if (a.persistent) {
-        // enough CTAs to fill the GPU once, shared out over the views in
-        // proportion to their estimated work (at least one CTA each)
-        int per_sm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
-        if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        const long long resident = static_cast<long long>(per_sm) * num_sms;
-        double sum = 0.0;
-        for (int u = 0; u < units; ++u) sum += uwork[u];
-        for (int u = 0; u < units; ++u) {
-            const double share = sum > 0.0 ? uwork[u] / sum : 1.0 / units;
-            const long long c = std::min(needed, std::max(1LL, static_cast<long long>(share * resident + 0.5)));
-            a.cta_begin[u] = static_cast<int>(total);
-            total += c;
-        }
-    } else {
-        for (int u = 0; u < units; ++u) {
-            a.cta_begin[u] = static_cast<int>(total);
-            total += needed;
-        }
-    }
+    const long long total = static_cast<long long>(units) * a.pk.blocks;
     if (total < 1 || total > 0x7fffffffLL) return cudaErrorInvalidValue;
-    a.cta_begin[units] = static_cast<int>(total);
     L.func = k;
     L.grid = dim3(static_cast<unsigned>(total));
-    L.block = dim3(threads);
+    L.block = dim3(32 * cfg.cta_warps);
     L.smem = smem;
     return cudaSuccess;
 }
 
-cudaError_t launch_march(MarchArgs &a, const LaunchCfg &cfg, int num_sms, const double *work, cudaStream_t stream)
+cudaError_t launch_march(MarchArgs &a, const LaunchCfg &cfg, cudaStream_t stream)
 {
     KernelLaunch L;
-    cudaError_t e = plan_march(a, cfg, num_sms, work, L);
+    cudaError_t e = plan_march(a, cfg, L);
     if (e != cudaSuccess) return e;
     void *params[] = {&a};
     return cudaLaunchKernel(L.func, L.grid, L.block, params, L.smem, stream);

@@ -74,7 +74,7 @@ struct gbd_ctx {
     gbd::GraphCache *graphs = nullptr;
     gbd::Server *server = nullptr;
     std::map<gbd::TuneKey, gbd::TuneEntry> tuned;
-    std::map<std::array<int, 4>, int *> tile_orders;  // device tables of tile_order(), by image and packet shape
+    std::map<std::array<int, 4>, int *> block_orders;  // device tables of block_order(), by image and block shape
     ~gbd_ctx();
     gbd::Volume *find(gbd_volume id);
 };
@@ -115,7 +115,6 @@ int check_launch(const LaunchCfg &c);
 // A batch of n views runs as march_chunks(n) launches; fill_args sets up the
 // arguments of launch c from the host view array hv.
 int march_chunks(int n);
-double view_work(const Volume &vol, const ViewDev &V, int width, int height);
 // Region schedule (see RegionArgs): slots per ray, 0 when it does not apply.
 int region_slots(const Volume &vol, const LaunchCfg &cfg, const gbd_image_spec &spec, int nreg[3], long long n_views);
 struct RegionPlan {
@@ -131,19 +130,16 @@ cudaError_t upload_region_tables(const RegionPlan &P, char *scratch, cudaStream_
 cudaError_t enqueue_regions(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, const RegionPlan &P,
                             const gbd_image_spec &spec, const LaunchCfg &cfg, float *dev_out, char *scratch,
                             cudaStream_t st, int *launches);
-std::vector<double> view_works(const Volume &vol, const std::vector<ViewDev> &hv, int width, int height);
 void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c, const gbd_image_spec &s,
-               float *out, uint32_t *samples, int *queue, const LaunchCfg &cfg, int *err_word);
+               float *out, uint32_t *samples, const LaunchCfg &cfg, int *err_word);
 // Time groups of a filled launch (batched renders; see MarchArgs).
 void group_views(MarchArgs &a, int gmax);
-// The order in which persistent warps take a view's tiles: by distance of the
-// tile from the image centre, nearest first (the longest rays of a centred
-// box first, so the launch ends on short ones).  A device table cached in the
-// context for up to 64 image geometries; NULL (counter order) beyond them or
-// if it cannot be made.  Used by launches of one
-// view or time group; with several, warps move on to the other views' tiles
-// instead, and counter order keeps neighbouring warps on neighbouring tiles.
-const int *tile_order(Ctx &ctx, int width, int height, int packet_w, int packet_h);
+// The order in which the CTAs of a launch of one view or time group take its
+// blocks: by distance of the block from the image centre, nearest first (the longest
+// rays of a centred box first, so the launch ends on short ones).  A device table cached
+// in the context for up to 64 image geometries; NULL (row order) beyond them or
+// if it cannot be made.  Launches of several views run view after view in row order.
+const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk);
 // Views, or time groups when grouped, of a filled launch.
 int launch_units(const MarchArgs &a);
 bool build_layout(const int n[3], int B, int S, std::vector<int32_t> &tab, long long &epoch_stride, int morton_cells);

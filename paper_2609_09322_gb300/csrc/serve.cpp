@@ -208,10 +208,12 @@ bool Server::launch_wave_from_queue(WaveSlot &w)
             d.view = r.view;
             d.width = r.spec.width;
             d.height = r.spec.height;
-            d.tiles_x = (r.spec.width + launch.packet_w - 1) / launch.packet_w;
-            d.tiles_y = (r.spec.height + launch.packet_h - 1) / launch.packet_h;
+            const PacketGrid pk =
+                packet_grid(r.spec.width, r.spec.height, launch.packet_w, launch.packet_h, launch.cta_warps);
+            a.pk = pk;  // packets and blocks: the same for every request
+            d.blocks_x = pk.blocks_x;
             d.cta_begin = cta_begin;
-            cta_begin += (d.tiles_x * d.tiles_y + launch.cta_warps - 1) / launch.cta_warps;
+            cta_begin += pk.blocks;
             if (r.spec.out_on_host) {
                 d.out = reinterpret_cast<float *>(d_img + img_off);
                 host_off[first + i] = img_off;
@@ -222,8 +224,6 @@ bool Server::launch_wave_from_queue(WaveSlot &w)
             }
         }
         a.n_reqs = static_cast<int>(cnt);
-        a.packet_w = launch.packet_w;
-        a.packet_h = launch.packet_h;
         a.total_ctas = cta_begin;
         a.error_word = ctx->err_word;
         e = launch_wave(a, launch, w.stream);

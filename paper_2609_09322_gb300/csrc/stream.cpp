@@ -180,9 +180,6 @@ extern "C" int gbd_render_streamed(gbd_ctx *ctx, const gbd_grid *grid, const gbd
     int slabs_done = 0, launches = 0;
     auto args = std::make_unique<MarchArgs>();
     std::vector<ViewDev> hv(static_cast<size_t>(n));
-    char *queue = nullptr;
-    const size_t qbytes = (static_cast<size_t>(n) * sizeof(int) + 255) / 256 * 256;
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&queue), qbytes * 2);
     for (int k = 0; k < n_slabs && e == cudaSuccess && rc == GBD_OK; ++k) {
         if (m0[k] > m1[k]) continue;  // no ray reaches a snapshot inside this slab
         SlabBuffer &b = buf[slabs_done % 2];
@@ -253,13 +250,10 @@ extern "C" int gbd_render_streamed(gbd_ctx *ctx, const gbd_grid *grid, const gbd
         for (int v = 0; v < n && rc == GBD_OK; ++v)
             rc = make_view(sv, views[v], spec->width, spec->height, spec->fov_u, spec->fov_v, hv[v]);
         if (rc != GBD_OK) break;
-        int *q = reinterpret_cast<int *>(queue + (slabs_done % 2) * qbytes);
-        if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, qbytes, rs);
-        const std::vector<double> work = view_works(sv, hv, spec->width, spec->height);
         for (int c = 0; c < march_chunks(n) && e == cudaSuccess; ++c) {
-            fill_args(*args, sv, hv.data(), n, c, *spec, spec->out, spec->samples, q, cfg, ctx->err_word);
+            fill_args(*args, sv, hv.data(), n, c, *spec, spec->out, spec->samples, cfg, ctx->err_word);
             args->accumulate = 1;
-            e = launch_march(*args, cfg, ctx->num_sms, work.data() + static_cast<size_t>(c) * kViewsPerLaunch, rs);
+            e = launch_march(*args, cfg, rs);
             ++launches;
         }
         if (e == cudaSuccess) e = cudaEventRecord(b.rendered, rs);
@@ -276,7 +270,6 @@ extern "C" int gbd_render_streamed(gbd_ctx *ctx, const gbd_grid *grid, const gbd
     if (e == cudaSuccess && bad) e = cudaMemcpy(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost);
     for (auto &b : buf) release(b);
     if (bad) cudaFree(bad);
-    if (queue) cudaFree(queue);
     if (rc != GBD_OK) return rc;
     if (e != cudaSuccess) return cuda_fail(e, "streamed render");
     if (h_bad)
@@ -331,14 +324,7 @@ extern "C" int gbd_render_labelled(gbd_ctx *ctx, const gbd_volume *vols, int32_t
     const size_t pix = static_cast<size_t>(spec->width) * spec->height * n;
     cudaError_t e = cudaMemsetAsync(spec->out, 0, pix * sizeof(float), st);
     if (e == cudaSuccess && spec->samples) e = cudaMemsetAsync(spec->samples, 0, pix * sizeof(uint32_t), st);
-    char *queue = nullptr;
-    const size_t qbytes = (static_cast<size_t>(n) * sizeof(int) + 255) / 256 * 256;
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void **>(&queue), qbytes * n_vols, st);
     if (e != cudaSuccess) return cuda_fail(e, "labelled render setup");
-    if ((e = cudaMemsetAsync(queue, 0, qbytes * n_vols, st)) != cudaSuccess) {
-        cudaFreeAsync(queue, st);
-        return cuda_fail(e, "labelled render setup");
-    }
     auto args = std::make_unique<MarchArgs>();
     std::vector<ViewDev> hv(static_cast<size_t>(n));
     int launches = 0;
@@ -359,18 +345,16 @@ extern "C" int gbd_render_labelled(gbd_ctx *ctx, const gbd_volume *vols, int32_t
         for (int v = 0; v < n && rc == GBD_OK; ++v)
             rc = make_view(*vs[k], views[v], spec->width, spec->height, spec->fov_u, spec->fov_v, hv[v]);
         if (rc != GBD_OK) break;
-        const std::vector<double> work = view_works(*vs[k], hv, spec->width, spec->height);
-        int *q = reinterpret_cast<int *>(queue + k * qbytes);
         cudaStream_t ks = side_by_side ? ctx->aux[k % 4] : st;
         if (side_by_side) e = cudaStreamWaitEvent(ks, start, 0);
         for (int c = 0; c < march_chunks(n) && e == cudaSuccess; ++c) {
             if (side_by_side) {
-                fill_args(*args, *vs[k], hv.data(), n, c, *spec, parts + pix * k, nullptr, q, cfg, ctx->err_word);
+                fill_args(*args, *vs[k], hv.data(), n, c, *spec, parts + pix * k, nullptr, cfg, ctx->err_word);
             } else {
-                fill_args(*args, *vs[k], hv.data(), n, c, *spec, spec->out, spec->samples, q, cfg, ctx->err_word);
+                fill_args(*args, *vs[k], hv.data(), n, c, *spec, spec->out, spec->samples, cfg, ctx->err_word);
                 args->accumulate = 1;
             }
-            e = launch_march(*args, cfg, ctx->num_sms, work.data() + static_cast<size_t>(c) * kViewsPerLaunch, ks);
+            e = launch_march(*args, cfg, ks);
             ++launches;
         }
         // side streams: the caller's stream waits for each sub-domain
@@ -400,10 +384,8 @@ extern "C" int gbd_render_labelled(gbd_ctx *ctx, const gbd_volume *vols, int32_t
     }
     if (parts) cudaFreeAsync(parts, st);
     if (start) cudaEventDestroy(start);
-    cudaError_t ef = cudaFreeAsync(queue, st);
     if (rc != GBD_OK) return rc;
     if (e != cudaSuccess) return cuda_fail(e, "labelled render");
-    if (ef != cudaSuccess) return cuda_fail(ef, "labelled render scratch");
     set_launch_count(launches);
     return GBD_OK;
 }

@@ -72,8 +72,7 @@ int time_config(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, con
     int nreg[3];
     const int slots = region_slots(vol, cfg, spec, nreg, n);
     const RegionPlan plan = slots > 0 ? region_plan(vol, cfg, spec, hv) : RegionPlan();
-    const size_t qbytes = slots > 0 ? plan.total : (static_cast<size_t>(n) * sizeof(int) + 255) / 256 * 256;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&scratch), qbytes, st);
+    cudaError_t e = slots > 0 ? cudaMallocAsync(reinterpret_cast<void **>(&scratch), plan.total, st) : cudaSuccess;
     if (e != cudaSuccess) return cuda_fail(e, "tune scratch");
     if (slots > 0) e = upload_region_tables(plan, scratch, st);
     cudaEvent_t a = nullptr, b = nullptr;
@@ -82,20 +81,16 @@ int time_config(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, con
     std::vector<float> times;
     auto args = std::make_unique<MarchArgs>();
     const int chunks = march_chunks(n);
-    const std::vector<double> work = view_works(vol, hv, spec.width, spec.height);
     for (int r = 0; r <= reps && e == cudaSuccess; ++r) {
-        e = slots > 0 ? cudaSuccess : cudaMemsetAsync(scratch, 0, qbytes, st);
-        if (e == cudaSuccess) e = cudaEventRecord(a, st);
+        e = cudaEventRecord(a, st);
         int launches = 0;
         if (slots > 0 && e == cudaSuccess)
             e = enqueue_regions(ctx, vol, hv, plan, spec, cfg, spec.out, scratch, st, &launches);
         for (int c = 0; c < chunks && e == cudaSuccess && slots == 0; ++c) {
-            fill_args(*args, vol, hv.data(), n, c, spec, spec.out, nullptr, reinterpret_cast<int *>(scratch), cfg,
-                      ctx.err_word);
+            fill_args(*args, vol, hv.data(), n, c, spec, spec.out, nullptr, cfg, ctx.err_word);
             group_views(*args, cfg.group);
-            if (cfg.persistent && launch_units(*args) == 1)
-                args->tile_order = tile_order(ctx, spec.width, spec.height, cfg.packet_w, cfg.packet_h);
-            e = launch_march(*args, cfg, ctx.num_sms, work.data() + static_cast<size_t>(c) * kViewsPerLaunch, st);
+            if (launch_units(*args) == 1) args->block_order = block_order(ctx, spec.width, spec.height, args->pk);
+            e = launch_march(*args, cfg, st);
         }
         if (e == cudaSuccess) e = cudaEventRecord(b, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(b);
@@ -105,7 +100,7 @@ int time_config(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, con
     }
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);
-    cudaFreeAsync(scratch, st);
+    if (scratch) cudaFreeAsync(scratch, st);
     if (e != cudaSuccess) return cuda_fail(e, "tune launch");
     std::sort(times.begin(), times.end());
     ms_out = times[times.size() / 2];
@@ -322,15 +317,6 @@ int gbd_tune(gbd_ctx *ctx, gbd_volume vid, const gbd_view *views, int32_t n, con
                             best = c;
                         }
                     }
-        LaunchCfg flat{8, 4, 8, 2, 0, 0, 0, kGroupDefault};
-        float ms = 0.f;
-        if ((rc = time_config(*ctx, *vol, hv, *spec, flat, st, 3, ms))) return rc;
-        report(flat, ms, vol->brick, vol->super_brick);
-        ++tried;
-        if (ms < best_ms) {
-            best_ms = ms;
-            best = flat;
-        }
         // region schedule, for batches of many views
         if (n >= 8) {
             const int regions[2] = {32, 64};
