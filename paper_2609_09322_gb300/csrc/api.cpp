@@ -1186,16 +1186,18 @@ int gbd_load_snapshots(gbd_ctx *ctx, const gbd_grid *grid, const gbd_fields *f, 
         e = cudaDeviceSynchronize();
         if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "wait for device inputs"); }
     }
-    e = cudaMemcpyAsync(vol->axis_off, tab.data(), tab_bytes, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(vol->rec, 0, bytes, st);
-    if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "volume init"); }
-
     const size_t esz = f->dtype_in == GBD_IN_F64 ? 8 : 4;
     const size_t ncell = static_cast<size_t>(g.n[0]) * g.n[1] * g.n[2];
+    e = cudaMemcpyAsync(vol->axis_off, tab.data(), tab_bytes, cudaMemcpyHostToDevice, st);
+    // the records that packing leaves alone (padding cells; the empty halves of paired
+    // blocks) are zero; without any, every record is written
+    if (e == cudaSuccess && (vol->paired || static_cast<size_t>(cells) != ncell))
+        e = cudaMemsetAsync(vol->rec, 0, bytes, st);
+    if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "volume init"); }
+
     char *stage = nullptr;
-    int *bad = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void **>(&bad), 256, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(bad, 0, 256, st);
+    int *bad = ctx->err_word + kLoadFlags;  // loads of a context are serialised by its lock
+    e = cudaMemsetAsync(bad, 0, 2 * sizeof(int), st);
     if (e == cudaSuccess && !f->on_device) e = cudaMallocAsync(reinterpret_cast<void **>(&stage), ncell * esz * 4, st);
     for (int m = 0; m < g.n_epochs && e == cudaSuccess; ++m) {
         const char *jsrc = static_cast<const char *>(f->j) + m * ncell * esz;
@@ -1229,7 +1231,6 @@ int gbd_load_snapshots(gbd_ctx *ctx, const gbd_grid *grid, const gbd_fields *f, 
     int h_bad[2] = {0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h_bad, bad, 2 * sizeof(int), cudaMemcpyDeviceToHost, st);
     if (stage) cudaFreeAsync(stage, st);
-    if (bad) cudaFreeAsync(bad, st);
     cudaError_t es = cudaStreamSynchronize(st);
     if (e == cudaSuccess) e = es;
     if (e != cudaSuccess) { cleanup(); return cuda_fail(e, "volume pack"); }

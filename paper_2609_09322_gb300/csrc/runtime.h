@@ -38,6 +38,10 @@ struct Volume {
 struct GraphCache;
 struct Server;
 
+// Words of gbd_ctx::err_word that a load uses: invalid values seen, and the
+// largest Gamma^2 of the stored records.
+constexpr int kLoadFlags = 32;
+
 // Autotuning class of a render: results are cached per key.
 struct TuneKey {
     int n[3];
@@ -70,7 +74,7 @@ struct gbd_ctx {
     // by side (each relies on its regions' records staying in L2), while a
     // batch's copy to host memory still overlaps the next batch's march.
     cudaEvent_t region_done = nullptr;
-    int *err_word = nullptr;          // bounds-check word of checked builds
+    int *err_word = nullptr;          // 256 bytes: bounds-check word of checked builds, load flags at kLoadFlags
     gbd::GraphCache *graphs = nullptr;
     gbd::Server *server = nullptr;
     std::map<gbd::TuneKey, gbd::TuneEntry> tuned;
