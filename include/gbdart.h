@@ -164,7 +164,8 @@ typedef struct {
 typedef struct {
     int32_t packet_w, packet_h;  /* pixels of one warp packet: 8x4, 4x8, 16x2, 32x1 */
     int32_t cta_warps;           /* warps per CTA: 1, 2, 4 or 8                     */
-    int32_t depth;               /* cells in flight per lane: 1, 2 or 4            */
+    int32_t depth;               /* cells gathered ahead per lane, while as many are
+                                    evaluated: 1, 2 or 4 (4 runs as 2)             */
     int32_t persistent;          /* accepted, 0 or 1, without effect: every launch
                                     is one packet per warp, view after view      */
     int32_t regcap;              /* 1 = kernel built for at most 80 registers/thread */

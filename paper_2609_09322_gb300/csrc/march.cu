@@ -19,9 +19,9 @@
 //     coordinate at the chord midpoint, the two snapshot records, the Doppler
 //     boost of each, their linear interpolation, and a compensated float32
 //     accumulation of value * ds.
-// Cells are gathered DEPTH at a time: the traversal runs ahead, all loads of
-// the group are issued, then the group is evaluated, so each lane keeps up to
-// 2 * DEPTH independent loads in flight.
+// Cells are gathered a stage of H at a time, while the stage before is being
+// evaluated (run_stages), so each lane keeps up to 4 H independent loads in
+// flight.
 //
 // Time groups (batched renders of one direction at several observer times):
 // one traversal per ray serves up to 4 or 8 views, each with its own sums
@@ -545,43 +545,35 @@ __device__ __forceinline__ int floor_plus1(float u, float &w)
     return static_cast<int>(static_cast<unsigned>(__float_as_int(t)) - 0x4B3FFFFFu);
 }
 
-// The march's loop.  A stage is H cells of every lane: gather() traverses them
-// and issues the loads of their records, evaluate() boosts and sums them.  PIPED: two
-// stages alternate, and each is evaluated after the next one has been gathered, so that
-// its loads have the evaluation of the stage before and the traversal of
-// the stage after to arrive in.  What bounds the march is waiting for its gathers (issue
-// slots half used); a lane has as many cells in flight as one that gathers 2 H
-// and then evaluates 2 H, but does not stand still for them (one 1024^2 image of 512^3 x 8
-// bfloat16/float16 records: 865 us with 4 cells gathered and evaluated, 809 as 2 + 2; region schedule
-// of 256 float32 views: 20.1 -> 19.4 ms).
-template <bool PIPED, class Stage, class Gather, class Evaluate>
+// The march's loop.  A stage is some cells of every lane: gather() traverses them
+// and issues the loads of their records, evaluate() boosts and sums them.  Two stages
+// alternate, and each is evaluated after the next one has been gathered, so that its loads
+// have the evaluation of the stage before and the traversal of the stage after to arrive
+// in.  What bounds the march is waiting for its gathers (issue slots half used).
+// Measured, cells gathered then evaluated / stages of one / of two (at most 80
+// registers each): 24 views of 384^2 of 256^3 x 16 float32 2.93 / 2.81 / 2.49 ms, one
+// 1024^2 image of 512^3 x 8 float32 1.50 / 1.44 / 1.41 ms, of paired
+// bfloat16/float16 records 0.87 / 0.96 / 0.82 ms.
+template <class Stage, class Gather, class Evaluate>
 __device__ __forceinline__ void run_stages(const bool &alive, Gather gather, Evaluate evaluate)
 {
-    Stage a;
-    if constexpr (PIPED) {
-        if (!__any_sync(kFull, alive)) return;
-        Stage b;
-        gather(a);
-        while (__any_sync(kFull, alive)) {
-            gather(b);
-            evaluate(a);
-            gather(a);
-            evaluate(b);
-        }
+    if (!__any_sync(kFull, alive)) return;
+    Stage a, b;
+    gather(a);
+    while (__any_sync(kFull, alive)) {
+        gather(b);
         evaluate(a);
-    } else {
-        while (__any_sync(kFull, alive)) {
-            gather(a);
-            evaluate(a);
-        }
+        gather(a);
+        evaluate(b);
     }
+    evaluate(a);
 }
 
 // The march of march_ray for bfloat16/float16 records (see the file
 // header): same cells, chords, midpoints and hat weights (Eqs. 2, 6-9, 19),
 // with the epoch coordinate of EpochLine.  PLAIN: the Doppler factor in the
 // plain form (volumes whose Gamma <= 8).
-template <int DEPTH, bool PAIRED, bool PARTIAL, bool PLAIN>
+template <int H, bool PAIRED, bool PARTIAL, bool PLAIN>
 __device__ __forceinline__ void march_ray_bf16(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
                                                int width, int height, float *out_img, uint32_t *cnt_img,
                                                int *err_word, const int32_t *__restrict__ tab, bool accumulate)
@@ -613,7 +605,6 @@ __device__ __forceinline__ void march_ray_bf16(const VolDev &vol, const ViewDev 
 
     float acc = 0.f;
     uint32_t count = 0;
-    constexpr int H = DEPTH > 1 ? DEPTH / 2 : 1;  // cells per stage (see run_stages)
     struct Stage {
         float wgt[H], dsv[H];
         bool has[H];
@@ -666,7 +657,7 @@ __device__ __forceinline__ void march_ray_bf16(const VolDev &vol, const ViewDev 
             count += T.has[d] ? 1u : 0u;
         }
     };
-    run_stages<(DEPTH > 1), Stage>(alive, gather, evaluate);
+    run_stages<Stage>(alive, gather, evaluate);
 
     if (in_image) {
         const long long pix = static_cast<long long>(q) * width + p;
@@ -709,7 +700,7 @@ struct ChanPtrs {
 // has ended takes no step and reads no record), with the exact Q31.32 epoch
 // coordinate, the records' own Doppler factor and compensated sums: float32
 // records, and the vector and memory-analysis forms of both stores.
-template <int STORE, int DEPTH, bool PAIRED, bool PARTIAL, int NCH, bool TOUCH>
+template <int STORE, int H, bool PAIRED, bool PARTIAL, int NCH, bool TOUCH>
 __device__ __forceinline__ void march_ray_exact(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
                                                 int width, int height, float *out_img, uint32_t *cnt_img,
                                                 int *err_word, const int32_t *__restrict__ tab, bool accumulate,
@@ -750,7 +741,6 @@ __device__ __forceinline__ void march_ray_exact(const VolDev &vol, const ViewDev
 #pragma unroll
     for (int c = 0; c < kNch; ++c) cacc[c] = ccomp[c] = 0.f;
 
-    constexpr int H = DEPTH > 1 ? DEPTH / 2 : 1;  // cells per stage (see run_stages)
     struct Stage {
         float wgt[H], dsv[H];
         bool has[H];
@@ -846,7 +836,7 @@ __device__ __forceinline__ void march_ray_exact(const VolDev &vol, const ViewDev
             }
         }
     };
-    run_stages<(DEPTH > 1), Stage>(alive, gather, evaluate);
+    run_stages<Stage>(alive, gather, evaluate);
     if (in_image && !TOUCH) {
         const long long pix = static_cast<long long>(q) * width + p;
         if (PARTIAL) {
@@ -866,7 +856,7 @@ __device__ __forceinline__ void march_ray_exact(const VolDev &vol, const ViewDev
     }
 }
 
-template <int STORE, int DEPTH, bool PAIRED, bool PARTIAL = false, int NCH = 0, bool TOUCH = false>
+template <int STORE, int H, bool PAIRED, bool PARTIAL = false, int NCH = 0, bool TOUCH = false>
 __device__ __forceinline__ void march_ray(const VolDev &vol, const ViewDev &V, const RayBox &B, int p, int q,
                                           int width, int height, float *out_img, uint32_t *cnt_img, int *err_word,
                                           const int32_t *__restrict__ tab, bool accumulate = false,
@@ -874,13 +864,13 @@ __device__ __forceinline__ void march_ray(const VolDev &vol, const ViewDev &V, c
 {
     if constexpr (STORE == GBD_STORE_BF16_F16U && NCH == 0 && !TOUCH) {
         if (vol.plain_boost)
-            march_ray_bf16<DEPTH, PAIRED, PARTIAL, true>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
+            march_ray_bf16<H, PAIRED, PARTIAL, true>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
                                                          tab, accumulate);
         else
-            march_ray_bf16<DEPTH, PAIRED, PARTIAL, false>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
+            march_ray_bf16<H, PAIRED, PARTIAL, false>(vol, V, B, p, q, width, height, out_img, cnt_img, err_word,
                                                           tab, accumulate);
     } else {
-        march_ray_exact<STORE, DEPTH, PAIRED, PARTIAL, NCH, TOUCH>(vol, V, B, p, q, width, height, out_img, cnt_img,
+        march_ray_exact<STORE, H, PAIRED, PARTIAL, NCH, TOUCH>(vol, V, B, p, q, width, height, out_img, cnt_img,
                                                                    err_word, tab, accumulate, ch);
     }
 }
@@ -1126,7 +1116,7 @@ __device__ __forceinline__ BlockWork block_work(const MarchArgs &a)
 
 // MINB = 1 leaves the register count to the compiler; MINB = 3 asks for
 // three 256-thread CTAs per SM (at most 80 registers per thread).
-template <int STORE, int DEPTH, int MINB, bool PAIRED>
+template <int STORE, int H, int MINB, bool PAIRED>
 __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_tab[];
@@ -1137,7 +1127,7 @@ __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant_
     const long long img = w.unit * (a.img_stride ? a.img_stride : static_cast<long long>(a.width) * a.height);
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
-    march_ray<STORE, DEPTH, PAIRED>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height, a.out + img,
+    march_ray<STORE, H, PAIRED>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height, a.out + img,
                                     a.samples ? a.samples + img : nullptr, a.error_word, s_tab, a.accumulate != 0);
 }
 
@@ -1172,9 +1162,10 @@ __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ M
 }
 
 // Vector renders: march_kernel's work split with NCH extra channels summed
-// along every ray (depth 2, the compiler's register budget).
-template <int STORE, int NCH, bool PAIRED, int MINB>
-__global__ void __launch_bounds__(256, MINB) vector_kernel(const __grid_constant__ MarchArgs a)
+// along every ray (stages of one cell, at most 96 registers: six views of 384^2 of
+// 192^3 x 8 with three channels 878 us at the compiler's 106, 854 at 96, 897 at 80).
+template <int STORE, int NCH, bool PAIRED>
+__global__ void __maxnreg__(96) vector_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_tab[];
     stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
@@ -1184,7 +1175,7 @@ __global__ void __launch_bounds__(256, MINB) vector_kernel(const __grid_constant
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
     const ChanPtrs ch{a.chan, a.chan_comp_stride, a.chan_cell_stride, nullptr};
-    march_ray<STORE, 2, PAIRED, false, NCH>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height,
+    march_ray<STORE, 1, PAIRED, false, NCH>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height,
                                             a.out + w.unit * a.img_stride, nullptr, a.error_word, s_tab, false, ch);
 }
 
@@ -1213,7 +1204,7 @@ __global__ void __launch_bounds__(256, 1) touch_kernel(const __grid_constant__ M
 // the largest volume of the launch); every ray runs the same march_ray as the
 // single-volume kernel, so a request's pixels are the same whether it is
 // served alone or in a mix.
-template <int DEPTH, int MINB>
+template <int H, int MINB>
 __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__ WaveArgs a)
 {
     extern __shared__ int32_t s_tab[];
@@ -1233,17 +1224,17 @@ __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__
     const RayBox box = grid_box(R.vol, R.view);
     if (R.vol.store == GBD_STORE_F32) {
         if (R.vol.paired)
-            march_ray<GBD_STORE_F32, DEPTH, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
+            march_ray<GBD_STORE_F32, H, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
                                                         a.error_word, s_tab);
         else
-            march_ray<GBD_STORE_F32, DEPTH, false>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
+            march_ray<GBD_STORE_F32, H, false>(R.vol, R.view, box, p, q, R.width, R.height, R.out, R.samples,
                                                          a.error_word, s_tab);
     } else {
         if (R.vol.paired)
-            march_ray<GBD_STORE_BF16_F16U, DEPTH, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
+            march_ray<GBD_STORE_BF16_F16U, H, true>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
                                                               R.samples, a.error_word, s_tab);
         else
-            march_ray<GBD_STORE_BF16_F16U, DEPTH, false>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
+            march_ray<GBD_STORE_BF16_F16U, H, false>(R.vol, R.view, box, p, q, R.width, R.height, R.out,
                                                                R.samples, a.error_word, s_tab);
     }
 }
@@ -1478,7 +1469,7 @@ __device__ __forceinline__ long long uniform(long long x)
 // spills: 32 warps per SM instead of 24.  256 views of a 384^3 x 32 float32 series: 19.49 ->
 // 18.99 ms (64 registers without it spill: 22.8).  The kernel is bound by what L2
 // delivers: with 2 and 4 times the gathers in flight (asynchronous copies into shared memory) it ran no faster.
-template <int STORE, int DEPTH, int MINB, bool PAIRED>
+template <int STORE, int H, int MINB, bool PAIRED>
 __global__ void __maxnreg__(MINB == 3 ? 64 : 128) region_kernel(const __grid_constant__ RegionArgs a)
 {
     extern __shared__ int32_t s_tab[];
@@ -1515,7 +1506,7 @@ __global__ void __maxnreg__(MINB == 3 ? 64 : 128) region_kernel(const __grid_con
     U.flags = uniform(V.flags);
     float *out = a.partial + static_cast<long long>(F.slot) * a.slot_stride +
                  static_cast<long long>(a.image[vi]) * a.width * a.height;
-    march_ray<STORE, DEPTH, PAIRED, true>(a.vol, U, F.B, static_cast<int>(pq & 0xffffu), static_cast<int>(pq >> 16),
+    march_ray<STORE, H, PAIRED, true>(a.vol, U, F.B, static_cast<int>(pq & 0xffffu), static_cast<int>(pq >> 16),
                                                 a.width, a.height, out, nullptr, a.error_word, s_tab);
 }
 
@@ -1539,13 +1530,15 @@ __global__ void __launch_bounds__(256) reduce_kernel(const __grid_constant__ Red
     }
 }
 
+// Stages of `depth` cells, at most two: four spill at 80 registers (1024^2 image of
+// bfloat16/float16 records 0.87 against 0.81 ms) or leave 16 warps per SM.
 template <int STORE, int MINB, bool PAIRED>
 void *select_depth(int depth)
 {
     switch (depth) {
     case 1: return reinterpret_cast<void *>(&march_kernel<STORE, 1, MINB, PAIRED>);
-    case 2: return reinterpret_cast<void *>(&march_kernel<STORE, 2, MINB, PAIRED>);
-    case 4: return reinterpret_cast<void *>(&march_kernel<STORE, 4, MINB, PAIRED>);
+    case 2:
+    case 4: return reinterpret_cast<void *>(&march_kernel<STORE, 2, MINB, PAIRED>);
     default: return nullptr;
     }
 }
@@ -1597,12 +1590,15 @@ void *select_kernel(int store, int depth, int capped, int paired)
     return nullptr;
 }
 
+// float32 stages of one cell whatever the depth: that march is bound by L2, and more
+// cells in flight only take registers (see region_kernel).  bfloat16/float16 stages of
+// two: 96 views of 192^2 of 256^3 x 16 1.90 -> 1.64 ms.
 template <int STORE, int MINB, bool PAIRED>
 void *select_region_depth(int depth)
 {
     switch (depth) {
     case 1: return reinterpret_cast<void *>(&region_kernel<STORE, 1, MINB, PAIRED>);
-    case 2: return reinterpret_cast<void *>(&region_kernel<STORE, 2, MINB, PAIRED>);
+    case 2: return reinterpret_cast<void *>(&region_kernel<STORE, STORE == GBD_STORE_F32 ? 1 : 2, MINB, PAIRED>);
     default: return nullptr;
     }
 }
@@ -1624,19 +1620,17 @@ void *select_region(int store, int depth, int capped, int paired)
     return nullptr;
 }
 
-template <int NCH, int MINB>
+template <int NCH>
 void *select_vector_store(int store, int paired)
 {
     if (store == GBD_STORE_F32)
-        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, true, MINB>)
-                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, false, MINB>);
+        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, true>)
+                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, false>);
     if (store == GBD_STORE_BF16_F16U)
-        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, true, MINB>)
-                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, false, MINB>);
+        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, true>)
+                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, false>);
     return nullptr;
 }
-
-
 
 void *select_wave(int depth, int capped)
 {
@@ -1667,17 +1661,12 @@ cudaError_t launch_wave(const WaveArgs &a, const LaunchCfg &cfg, cudaStream_t st
 
 cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, cudaStream_t stream)
 {
-    // the compiler's register budget: capped, the three-channel kernel spills
-    // and runs slower than the extra resident warps gain
-    void *k = n_chan == 1 ? select_vector_store<1, 1>(a.vol.store, a.vol.paired)
-                          : (n_chan == 3 ? select_vector_store<3, 1>(a.vol.store, a.vol.paired) : nullptr);
+    void *k = n_chan == 1 ? select_vector_store<1>(a.vol.store, a.vol.paired)
+                          : (n_chan == 3 ? select_vector_store<3>(a.vol.store, a.vol.paired) : nullptr);
     if (!k) return cudaErrorInvalidValue;
-    // grid as planned for the scalar kernel of the same budget
-    LaunchCfg c = cfg;
-    c.depth = 2;
-    c.regcap = 0;
+    // grid and shared memory as planned for the scalar kernel
     KernelLaunch L;
-    cudaError_t e = plan_march(a, c, L);
+    cudaError_t e = plan_march(a, cfg, L);
     if (e != cudaSuccess) return e;
     if (L.smem > 48 * 1024) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, L.smem);
