@@ -322,6 +322,44 @@ int march_chunks(int n) { return (n + kViewsPerLaunch - 1) / kViewsPerLaunch; }
 
 // Launch arguments of chunk c of a batch of n views: views c K .. c K + K - 1
 // (K = kViewsPerLaunch) and their images.
+// Two views have the same rays when every per-view constant but the epoch
+// coordinate at the image plane, the window and the prefactor agrees: the
+// same image plane, direction, grid frame, epoch rate per face and boost.
+static bool same_rays(const ViewDev &x, const ViewDev &y)
+{
+    return std::memcmp(x.g0, y.g0, sizeof(x.g0)) == 0 && std::memcmp(x.gu, y.gu, sizeof(x.gu)) == 0 &&
+           std::memcmp(x.gv, y.gv, sizeof(x.gv)) == 0 && std::memcmp(x.du, y.du, sizeof(x.du)) == 0 &&
+           std::memcmp(x.a_hi, y.a_hi, sizeof(x.a_hi)) == 0 && std::memcmp(x.a_lo, y.a_lo, sizeof(x.a_lo)) == 0 &&
+           std::memcmp(x.inv_a, y.inv_a, sizeof(x.inv_a)) == 0 && std::memcmp(x.w_hi, y.w_hi, sizeof(x.w_hi)) == 0 &&
+           std::memcmp(x.w_lo, y.w_lo, sizeof(x.w_lo)) == 0 && std::memcmp(&x.kk_hi, &y.kk_hi, sizeof(float)) == 0 &&
+           std::memcmp(&x.kk_lo, &y.kk_lo, sizeof(float)) == 0 && std::memcmp(x.sh_hi, y.sh_hi, sizeof(x.sh_hi)) == 0 &&
+           std::memcmp(x.sh_lo, y.sh_lo, sizeof(x.sh_lo)) == 0 && std::memcmp(&x.expo, &y.expo, sizeof(float)) == 0 &&
+           x.flags == y.flags;
+}
+
+// Which units a launch takes side by side, block by block: consecutive views (or
+// time groups, by their references) with the same rays whose observer times lie less
+// than two snapshots from one to the next.  At every cell such neighbours read a common
+// snapshot, which the second then finds in a cache; further apart or along other rays
+// they share no record.  18 float32 images of 512^2 of a 256^3 x 16 series, one after
+// the other / side by side: lone marches 860 / 833 us, groups of three 583 / 549.
+static void set_runs(MarchArgs &a)
+{
+    const int units = a.n_groups > 0 ? a.n_groups : a.n_views;
+    auto view = [&](int u) -> const ViewDev & { return a.views[a.n_groups > 0 ? a.group_ref[u] : u]; };
+    for (int u = 0; u < units;) {
+        int e = u + 1;
+        while (e < units && same_rays(view(u), view(e)) &&
+               std::llabs(view(e).u_obs - view(e - 1).u_obs) < (2LL << 32))
+            ++e;
+        for (int k = u; k < e; ++k) {
+            a.run_first[k] = static_cast<short>(u);
+            a.run_len[k] = static_cast<short>(e - u);
+        }
+        u = e;
+    }
+}
+
 void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c, const gbd_image_spec &s,
                float *out, uint32_t *samples, const LaunchCfg &cfg, int *err_word)
 {
@@ -338,21 +376,7 @@ void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c,
     a.samples = samples ? samples + img : nullptr;
     a.error_word = err_word;
     std::memcpy(a.views, hv + first, sizeof(ViewDev) * static_cast<size_t>(cnt));
-}
-
-// Two views have the same rays when every per-view constant but the epoch
-// coordinate at the image plane, the window and the prefactor agrees: the
-// same image plane, direction, grid frame, epoch rate per face and boost.
-static bool same_rays(const ViewDev &x, const ViewDev &y)
-{
-    return std::memcmp(x.g0, y.g0, sizeof(x.g0)) == 0 && std::memcmp(x.gu, y.gu, sizeof(x.gu)) == 0 &&
-           std::memcmp(x.gv, y.gv, sizeof(x.gv)) == 0 && std::memcmp(x.du, y.du, sizeof(x.du)) == 0 &&
-           std::memcmp(x.a_hi, y.a_hi, sizeof(x.a_hi)) == 0 && std::memcmp(x.a_lo, y.a_lo, sizeof(x.a_lo)) == 0 &&
-           std::memcmp(x.inv_a, y.inv_a, sizeof(x.inv_a)) == 0 && std::memcmp(x.w_hi, y.w_hi, sizeof(x.w_hi)) == 0 &&
-           std::memcmp(x.w_lo, y.w_lo, sizeof(x.w_lo)) == 0 && std::memcmp(&x.kk_hi, &y.kk_hi, sizeof(float)) == 0 &&
-           std::memcmp(&x.kk_lo, &y.kk_lo, sizeof(float)) == 0 && std::memcmp(x.sh_hi, y.sh_hi, sizeof(x.sh_hi)) == 0 &&
-           std::memcmp(x.sh_lo, y.sh_lo, sizeof(x.sh_lo)) == 0 && std::memcmp(&x.expo, &y.expo, sizeof(float)) == 0 &&
-           x.flags == y.flags;
+    set_runs(a);
 }
 
 // Time groups: each run of consecutive views with the same rays is cut into
@@ -422,6 +446,7 @@ void group_views(MarchArgs &a, int gmax)
     }
     a.group_size = most <= 4 ? 4 : kGroupMax;
     a.group_snaps = widest <= (static_cast<long long>(kGroupSnapsMin - 2) << 32) ? kGroupSnapsMin : kGroupSnapsMax;
+    set_runs(a);
 }
 
 int launch_units(const MarchArgs &a) { return a.n_groups > 0 ? a.n_groups : a.n_views; }

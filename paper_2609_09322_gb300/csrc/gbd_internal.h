@@ -141,6 +141,9 @@ struct MarchArgs {
     int group_ref[kViewsPerLaunch];        // the group's reference view: the largest u_obs
     float group_win[kViewsPerLaunch][2];   // the union of the members' windows
     long long view_delta[kViewsPerLaunch]; // u_obs of the view minus that of its group's reference, Q31.32
+    // units (views, or time groups) that the launch takes side by side: unit u is in the
+    // run of run_len[u] units from run_first[u]
+    short run_first[kViewsPerLaunch], run_len[kViewsPerLaunch];
     int accumulate;           // add to out (and samples) instead of storing
     float *out;               // n_views * width * height floats
     uint32_t *samples;        // optional, same shape
