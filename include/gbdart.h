@@ -186,11 +186,12 @@ typedef struct {
     int32_t group;               /* batches: time groups.  Consecutive views that
                                     differ only in observer time (same image plane,
                                     direction and grid frame; t_obs, and with it the
-                                    window, and nu_ratio free) and lie within three
-                                    snapshots of each other are marched together,
-                                    up to `group` per ray: one traversal and one
-                                    gather of the snapshots they share, one sum per
-                                    view.  0 = the default, 4; 1 = every view on its
+                                    window, and nu_ratio free) and lie within
+                                    min(3, (M + 1) / 2) snapshots of each other are
+                                    marched together, up to `group` per ray: one
+                                    traversal and one gather of the snapshots they
+                                    share, one sum per view (not in batches where
+                                    that would gather fewer than 7 views in 4 groups).  0 = the default, 4; 1 = every view on its
                                     own; at most 8.  A grouped view agrees with its
                                     lone render to FP32 rounding, not bitwise.       */
 } gbd_launch;

@@ -379,16 +379,21 @@ void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c,
     set_runs(a);
 }
 
-// Time groups: each run of consecutive views with the same rays is cut into
-// near-equal groups of at most gmax views, as few as keep the observer times
-// within a group close enough: within kGroupSnapsMax - 2 snapshots, so that its
-// members share the snapshots they read, and within half of a view's own
-// window of M + 1 snapshots, so that the shared march covers little that only
-// some members see.  Views farther apart march on their own: where members
-// share no snapshot a group saves only the traversal, and measured slower than the lone march for
-// float32 records (194 against 208 Gcell-samples/s on the 18-image series).
-// n_groups stays 0 (every view marched on its own) when gmax < 2 or no group
-// holds two views.
+// Time groups: each run of consecutive views with the same rays is cut into as few
+// groups of at most gmax views as keep the observer times within each group close
+// enough, near-equal in size where that takes no more of them: within
+// kGroupSnapsMax - 2 snapshots, so that its members share the snapshots they
+// read, and within half of a view's own window of M + 1 snapshots, so that the
+// shared march covers little that only some members see.  A view farther than that
+// from its neighbours marches on its own, and the others' groups do not depend on
+// it (24 float32 images of 384^2 of a 256^3 x 32 series, 23 of them 0.1 snapshots
+// apart and one late: 24 lone marches 1097 us, seven groups 571).
+// A view alone in a launch of groups costs the group kernel's set of snapshots: 1.6
+// (float32) to 1.8 (bfloat16/float16) lone marches where the spans are wide, so
+// groups are taken only where they hold 7/4 views on average (the same 24 views at
+// random times in random order, bfloat16/float16: in 18 groups 1297 us, alone 763).
+// n_groups stays 0 (every view marched on its own) when gmax < 2, below that, or
+// where no group holds two views.
 void group_views(MarchArgs &a, int gmax)
 {
     a.n_groups = 0;
@@ -397,41 +402,44 @@ void group_views(MarchArgs &a, int gmax)
     // Q31.32
     const long long span_max =
         std::min(static_cast<long long>(kGroupSnapsMax - 2) << 32, static_cast<long long>(a.vol.M + 1) << 31);
-    // observer times of views v0 .. v1 - 1 (all within 1e8 snapshots of zero, make_view: no overflow)
-    auto span = [&](int v0, int v1) {
-        long long lo = a.views[v0].u_obs, hi = lo;
-        for (int v = v0 + 1; v < v1; ++v) {
-            lo = std::min(lo, a.views[v].u_obs);
-            hi = std::max(hi, a.views[v].u_obs);
-        }
-        return hi - lo;
-    };
     int ng = 0;
     bool shared = false;
-    long long widest = 0;
     for (int v = 0; v < a.n_views;) {
-        int e = v + 1;
-        while (e < a.n_views && same_rays(a.views[v], a.views[e])) ++e;
-        const int len = e - v;
-        int parts = (len + gmax - 1) / gmax;
-        for (; parts < len; ++parts) {
-            bool fits = true;
-            for (int k = 0; k < parts && fits; ++k)
-                fits = span(v + len * k / parts, v + len * (k + 1) / parts) <= span_max;
-            if (fits) break;
+        int end = v + 1;
+        while (end < a.n_views && same_rays(a.views[v], a.views[end])) ++end;
+        // reach[i]: a group that starts with view i holds at most views i .. reach[i] - 1;
+        // need[i]: groups that views i .. end - 1 take.  A part of a group is a group,
+        // so taking each as long as it may be is the fewest.
+        // (observer times within 1e8 snapshots of zero, make_view: no overflow)
+        int reach[kViewsPerLaunch], need[kViewsPerLaunch + 1];
+        need[end] = 0;
+        for (int i = end - 1; i >= v; --i) {
+            long long lo = a.views[i].u_obs, hi = lo;
+            int e = i + 1;
+            for (; e < end && e - i < gmax; ++e) {
+                lo = std::min(lo, a.views[e].u_obs);
+                hi = std::max(hi, a.views[e].u_obs);
+                if (hi - lo > span_max) break;
+            }
+            reach[i] = e;
+            need[i] = 1 + need[e];
         }
-        for (int k = 0; k < parts; ++k) a.group_first[ng++] = v + len * k / parts;
-        shared = shared || parts < len;
-        v = e;
+        while (v < end) {
+            int e = std::min(reach[v], v + std::max(1, (end - v) / need[v]));
+            while (need[e] >= need[v]) ++e;  // reach[v] at the latest
+            a.group_first[ng++] = v;
+            shared = shared || e > v + 1;
+            v = e;
+        }
     }
     a.group_first[ng] = a.n_views;
-    if (!shared) return;
+    if (!shared || 7 * ng > 4 * a.n_views) return;
     a.n_groups = ng;
     int most = 1;
+    long long widest = 0;
     for (int g = 0; g < ng; ++g) {
         const int v0 = a.group_first[g], v1 = a.group_first[g + 1];
         most = std::max(most, v1 - v0);
-        widest = std::max(widest, span(v0, v1));
         int ref = v0;
         float lo = a.views[v0].win_lo, hi = a.views[v0].win_hi;
         for (int v = v0 + 1; v < v1; ++v) {
@@ -442,7 +450,10 @@ void group_views(MarchArgs &a, int gmax)
         a.group_ref[g] = ref;
         a.group_win[g][0] = lo;
         a.group_win[g][1] = hi;
-        for (int v = v0; v < v1; ++v) a.view_delta[v] = a.views[v].u_obs - a.views[ref].u_obs;
+        for (int v = v0; v < v1; ++v) {
+            a.view_delta[v] = a.views[v].u_obs - a.views[ref].u_obs;
+            widest = std::max(widest, -a.view_delta[v]);
+        }
     }
     a.group_size = most <= 4 ? 4 : kGroupMax;
     a.group_snaps = widest <= (static_cast<long long>(kGroupSnapsMin - 2) << 32) ? kGroupSnapsMin : kGroupSnapsMax;
