@@ -391,7 +391,7 @@ void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c,
 // A view alone in a launch of groups costs the group kernel's set of snapshots: 1.6
 // (float32) to 1.8 (bfloat16/float16) lone marches where the spans are wide, so
 // groups are taken only where they hold 7/4 views on average (the same 24 views at
-// random times in random order, bfloat16/float16: in 18 groups 1297 us, alone 763).
+// random times in random order, bfloat16/float16: in 20 groups 1297 us, alone 763).
 // n_groups stays 0 (every view marched on its own) when gmax < 2, below that, or
 // where no group holds two views.
 void group_views(MarchArgs &a, int gmax)

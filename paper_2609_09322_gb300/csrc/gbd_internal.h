@@ -50,6 +50,10 @@ __host__ __device__ inline int march_table_base(const int n[3], int axis)
     return axis == 0 ? 0 : (axis == 1 ? 2 * (n[0] + 1) : 2 * (n[0] + 1) + 2 * (n[1] + 1));
 }
 __host__ __device__ inline int march_table_entries(const int n[3]) { return 2 * (n[0] + n[1] + n[2] + 3); }
+// Shared memory of a march's CTA: the tables, after the spans of them that the rays
+// of its warps (8 at most) read.
+constexpr int kSpanEntries = 8 * 6;
+__host__ __device__ inline int staged_entries(const int n[3]) { return kSpanEntries + march_table_entries(n); }
 
 // Bits of ViewDev::flags above the public GBD_BEAMING / GBD_LOOKBACK bits:
 // axis i is mirrored (the view's direction has s_hat_i < 0).

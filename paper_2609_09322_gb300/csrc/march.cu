@@ -247,12 +247,6 @@ __device__ __forceinline__ int32_t tab_at(const int32_t *base, uint32_t cur)
     return *reinterpret_cast<const int32_t *>(reinterpret_cast<const char *>(base) + cur);
 }
 
-// Copies a volume's march tables into shared memory.
-__device__ __forceinline__ void stage_tables(int32_t *s_tab, const int32_t *src, int ntab)
-{
-    for (int i = threadIdx.x; i < ntab; i += blockDim.x) s_tab[i] = src[i];
-}
-
 // State of one axis of a ray: the next face crossing and what changes there.
 struct AxisState {
     float nkf;      // planes from the anchor cell's lower face to the next crossing
@@ -284,6 +278,88 @@ __device__ __forceinline__ RayBox grid_box(const VolDev &vol, const ViewDev &V)
         B.cur0[i] = 4u * static_cast<uint32_t>(march_table_base(vol.n, i) + (mirrored ? vol.n[i] + 1 : 0));
     }
     return B;
+}
+
+// Copies a volume's march tables into shared memory.
+__device__ __forceinline__ void stage_all(int32_t *s_tab, const VolDev &vol)
+{
+    const int total = march_table_entries(vol.n);
+    for (int i = threadIdx.x; i < total; i += blockDim.x) s_tab[i] = vol.mtab[i];
+    __syncthreads();
+}
+
+// The same for tables that take a thread more than kCopiesMax loads, only where the
+// rays of this CTA can read them (pixel (p, q) of this lane, as view V sees them,
+// within [win_lo, win_hi]): of each axis the table of the view's direction, from
+// the lowest cell that a ray enters to the highest.  s_tab stands after kSpanEntries words.
+// Per ray the cells follow from the float chord through the box: the march starts in
+// the cell of the later of s_in and win_lo, which set-up computes alike, and leaves
+// the box by s_out, so they are known to within float rounding (a few 2^-24 of the
+// largest coordinate in the sum; the slack is 2 and 2^-20 of it), and it reads at
+// most two entries past its last one.  A ray that misses the box or the window takes
+// no step; its lane may read an entry that is not there, and uses nothing of it.
+//
+// What it is for: a CTA marches 32 to 256 rays, and where an axis is long and the
+// rays are short or miss, copying everything takes longer than they do: 1024^2 images of
+// 4096 x 16 x 16 across the long axis 123 -> 40 us, filled by rays of 16 cells 167 -> 102.
+// Shorter tables are copied whole, as finding the spans takes about as long (32^3: 5% more).
+// A call, not inlined: the marches behind it keep their registers.
+constexpr int kCopiesMax = 32;
+__device__ __noinline__ void stage_spans(int32_t *s_tab, const VolDev &vol, const ViewDev &V, int p, int q, bool in_image,
+                                         float win_lo, float win_hi)
+{
+    const int threads = static_cast<int>(blockDim.x), t = static_cast<int>(threadIdx.x);
+    float g[3], s_in = -3.0e38f, s_out = 3.0e38f;
+    bool hit = in_image;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const long long gx = V.g0[i] + static_cast<long long>(p) * V.gu[i] + static_cast<long long>(q) * V.gv[i];
+        g[i] = fix_to_float(gx, kInv2p40);
+        if (V.inv_a[i] != 0.f) {
+            s_in = fmaxf(s_in, -g[i] * V.inv_a[i]);
+            // late by more than g's rounding, which a slowly crossed axis turns into a long way
+            const float n = static_cast<float>(vol.n[i]);
+            s_out = fminf(s_out, (n - g[i] + 1e-6f * (n + fabsf(g[i]))) * V.inv_a[i]);
+        } else if (gx < 0 || gx >= (static_cast<long long>(vol.n[i]) << 40)) {
+            hit = false;
+        }
+    }
+    // the test of setup_ray, twice as wide
+    s_in = fmaxf(s_in, win_lo);
+    if (!(fminf(s_out, win_hi) > s_in - 2e-3f * (1.f + fabsf(s_in)))) hit = false;
+    int32_t *s_span = s_tab - kSpanEntries;  // per warp: lowest and highest entry of each axis
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float n = static_cast<float>(vol.n[i]), from = s_in * V.a_hi[i], to = fmaxf(s_in, s_out) * V.a_hi[i];
+        const float slack = 2.0f + 1e-6f * (fabsf(g[i]) + fmaxf(fabsf(from), fabsf(to)));
+        const int first = static_cast<int>(fminf(fmaxf(g[i] + from - slack, 0.f), n));
+        const int last = static_cast<int>(fminf(fmaxf(g[i] + to + slack + 2.0f, 0.f), n));
+        const int lo = __reduce_min_sync(kFull, hit ? first : vol.n[i]);
+        const int hi = __reduce_max_sync(kFull, hit ? last : -1);
+        if ((t & 31) == 0) {
+            s_span[6 * (t >> 5) + 2 * i] = lo;
+            s_span[6 * (t >> 5) + 2 * i + 1] = hi;
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int i = 0; i < 3; ++i) {
+        int lo = vol.n[i], hi = -1;
+        for (int w = 0; w < threads >> 5; ++w) {
+            lo = min(lo, s_span[6 * w + 2 * i]);
+            hi = max(hi, s_span[6 * w + 2 * i + 1]);
+        }
+        // 0 <= lo <= n, hi <= n; no ray hits: lo = n, hi = -1
+        const int base = march_table_base(vol.n, i) + ((V.flags & (kFlagMirror0 << i)) != 0u ? vol.n[i] + 1 : 0);
+        for (int e = lo + t; e <= hi; e += threads) s_tab[base + e] = vol.mtab[base + e];
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ void stage_tables(int32_t *s_tab, const VolDev &vol, const ViewDev &V, int p, int q,
+                                             bool in_image, float win_lo, float win_hi)
+{
+    if (march_table_entries(vol.n) <= kCopiesMax * static_cast<int>(blockDim.x)) stage_all(s_tab, vol);
+    else stage_spans(s_tab, vol, V, p, q, in_image, win_lo, win_hi);
 }
 
 // State of a ray during the march: per axis the next crossing, the layout
@@ -1131,14 +1207,14 @@ __device__ __forceinline__ BlockWork block_work(const MarchArgs &a)
 template <int STORE, int H, int MINB, bool PAIRED>
 __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant__ MarchArgs a)
 {
-    extern __shared__ int32_t s_tab[];
-    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
-    __syncthreads();
+    extern __shared__ int32_t s_mem[];
+    int32_t *s_tab = s_mem + kSpanEntries;
     const BlockWork w = block_work<true>(a);
     const ViewDev &V = a.views[w.unit];
     const long long img = w.unit * (a.img_stride ? a.img_stride : static_cast<long long>(a.width) * a.height);
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    stage_tables(s_tab, a.vol, V, p, q, p < a.width && q < a.height, V.win_lo, V.win_hi);
     march_ray<STORE, H, PAIRED>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height, a.out + img,
                                     a.samples ? a.samples + img : nullptr, a.error_word, s_tab, a.accumulate != 0);
 }
@@ -1146,12 +1222,14 @@ __global__ void __launch_bounds__(256, MINB) march_kernel(const __grid_constant_
 // Time groups: march_kernel's work split over groups of views instead of
 // single views (group g is views group_first[g] .. group_first[g + 1] - 1).
 // DEPTH cells per iteration, S snapshots per cell, at most 80 registers.
-template <int STORE, int DEPTH, int G, int S>
+// SPANS: with tables too long to be copied whole (stage_spans).  A kernel of its own: the
+// call costs the others registers (bfloat16/float16 series of 18 images 434 -> 491 us).
+template <int STORE, int DEPTH, int G, int S, bool SPANS>
 __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ MarchArgs a)
 {
-    extern __shared__ int32_t s_tab[];
-    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
-    __syncthreads();
+    extern __shared__ int32_t s_mem[];
+    int32_t *s_tab = s_mem + kSpanEntries;
+    if constexpr (!SPANS) stage_all(s_tab, a.vol);
     const BlockWork w = block_work<STORE == GBD_STORE_F32>(a);
     const int first = a.group_first[w.unit];
     const int gcnt = a.group_first[w.unit + 1] - first;
@@ -1159,6 +1237,8 @@ __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ M
     const long long stride = a.img_stride ? a.img_stride : static_cast<long long>(a.width) * a.height;
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    if constexpr (SPANS)
+        stage_spans(s_tab, a.vol, V, p, q, p < a.width && q < a.height, a.group_win[w.unit][0], a.group_win[w.unit][1]);
     auto march = [&](auto plain) {
         march_group<STORE, DEPTH, G, S, decltype(plain)::value>(
             a.vol, V, a.group_win[w.unit][0], a.group_win[w.unit][1], a.views + first, a.view_delta + first, gcnt,
@@ -1179,13 +1259,13 @@ __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ M
 template <int STORE, int NCH, bool PAIRED>
 __global__ void __maxnreg__(96) vector_kernel(const __grid_constant__ MarchArgs a)
 {
-    extern __shared__ int32_t s_tab[];
-    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
-    __syncthreads();
+    extern __shared__ int32_t s_mem[];
+    int32_t *s_tab = s_mem + kSpanEntries;
     const BlockWork w = block_work<false>(a);
     const ViewDev &V = a.views[w.unit];
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    stage_tables(s_tab, a.vol, V, p, q, p < a.width && q < a.height, V.win_lo, V.win_hi);
     const ChanPtrs ch{a.chan, a.chan_comp_stride, a.chan_cell_stride, nullptr};
     march_ray<STORE, 1, PAIRED, false, NCH>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height,
                                             a.out + w.unit * a.img_stride, nullptr, a.error_word, s_tab, false, ch);
@@ -1197,13 +1277,13 @@ template <int STORE, bool PAIRED>
 __global__ void __launch_bounds__(256, 1) touch_kernel(const __grid_constant__ MarchArgs a, uint32_t *bits,
                                                         long long cells)
 {
-    extern __shared__ int32_t s_tab[];
-    stage_tables(s_tab, a.vol.mtab, march_table_entries(a.vol.n));
-    __syncthreads();
+    extern __shared__ int32_t s_mem[];
+    int32_t *s_tab = s_mem + kSpanEntries;
     const BlockWork w = block_work<false>(a);
     const ViewDev &V = a.views[w.unit];
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
+    stage_tables(s_tab, a.vol, V, p, q, p < a.width && q < a.height, V.win_lo, V.win_hi);
     const ChanPtrs ch{nullptr, 0, cells, bits};
     march_ray<STORE, 1, PAIRED, false, 0, true>(a.vol, V, grid_box(a.vol, V), p, q, a.width, a.height, a.out, nullptr,
                                                 a.error_word, s_tab, false, ch);
@@ -1219,7 +1299,8 @@ __global__ void __launch_bounds__(256, 1) touch_kernel(const __grid_constant__ M
 template <int H, int MINB>
 __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__ WaveArgs a)
 {
-    extern __shared__ int32_t s_tab[];
+    extern __shared__ int32_t s_mem[];
+    int32_t *s_tab = s_mem + kSpanEntries;
     const int b = static_cast<int>(blockIdx.x);
     int lo = 0, hi = a.n_reqs - 1;  // last request whose first CTA is <= b
     while (lo < hi) {
@@ -1228,11 +1309,9 @@ __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__
         else hi = mid - 1;
     }
     const ReqDev &R = a.reqs[lo];
-    const int ntab = march_table_entries(R.vol.n);
-    stage_tables(s_tab, R.vol.mtab, ntab);
-    __syncthreads();
     int p, q;
     block_pixel(a.pk, R.blocks_x, b - R.cta_begin, p, q);
+    stage_tables(s_tab, R.vol, R.view, p, q, p < R.width && q < R.height, R.view.win_lo, R.view.win_hi);
     const RayBox box = grid_box(R.vol, R.view);
     if (R.vol.store == GBD_STORE_F32) {
         if (R.vol.paired)
@@ -1564,8 +1643,8 @@ void *select_cap(int depth, int capped)
 template <int STORE, int DEPTH, int G>
 void *select_group_snaps(int snaps)
 {
-    if (snaps == kGroupSnapsMin) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, G, kGroupSnapsMin>);
-    if (snaps == kGroupSnapsMax) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, G, kGroupSnapsMax>);
+    if (snaps == kGroupSnapsMin) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, G, kGroupSnapsMin, false>);
+    if (snaps == kGroupSnapsMax) return reinterpret_cast<void *>(&group_kernel<STORE, DEPTH, G, kGroupSnapsMax, false>);
     return nullptr;
 }
 
@@ -1582,9 +1661,14 @@ void *select_group_size(int size, int snaps)
 // bfloat16/float16 ones at most two: a cell's S gathers already keep as many
 // loads in flight, and more cells' records would cost more warps than the
 // loads gain.
-void *select_group(int store, int size, int depth, int snaps)
+// Long tables (spans): one kernel per store, for any group.
+void *select_group(int store, int size, int depth, int snaps, bool spans)
 {
     if (depth != 1 && depth != 2 && depth != 4) return nullptr;
+    if (spans)
+        return store == GBD_STORE_F32
+                   ? reinterpret_cast<void *>(&group_kernel<GBD_STORE_F32, 1, kGroupMax, kGroupSnapsMax, true>)
+                   : reinterpret_cast<void *>(&group_kernel<GBD_STORE_BF16_F16U, 1, kGroupMax, kGroupSnapsMax, true>);
     if (store == GBD_STORE_F32) return select_group_size<GBD_STORE_F32, 1>(size, snaps);
     if (store == GBD_STORE_BF16_F16U)
         return depth == 1 ? select_group_size<GBD_STORE_BF16_F16U, 1>(size, snaps)
@@ -1661,7 +1745,7 @@ cudaError_t launch_wave(const WaveArgs &a, const LaunchCfg &cfg, cudaStream_t st
     // shared memory for the largest march tables of the launch
     int smem = 0;
     for (int r = 0; r < a.n_reqs; ++r)
-        smem = std::max(smem, static_cast<int>(sizeof(int32_t)) * march_table_entries(a.reqs[r].vol.n));
+        smem = std::max(smem, static_cast<int>(sizeof(int32_t)) * staged_entries(a.reqs[r].vol.n));
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
@@ -1749,7 +1833,8 @@ cudaError_t plan_march(const MarchArgs &a, const LaunchCfg &cfg, KernelLaunch &L
 {
     // n_groups > 0: time groups, one image's blocks of CTAs per group; else per view
     const bool grouped = a.n_groups > 0;
-    void *k = grouped ? select_group(a.vol.store, a.group_size, cfg.depth, a.group_snaps)
+    void *k = grouped ? select_group(a.vol.store, a.group_size, cfg.depth, a.group_snaps,
+                                     march_table_entries(a.vol.n) > kCopiesMax * 32 * cfg.cta_warps)
                       : select_kernel(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired);
     if (!k || a.n_views < 1 || a.n_views > kViewsPerLaunch) return cudaErrorInvalidValue;
     if (grouped && (a.n_groups > a.n_views || a.group_first[0] != 0 || a.group_first[a.n_groups] != a.n_views))
@@ -1760,7 +1845,7 @@ cudaError_t plan_march(const MarchArgs &a, const LaunchCfg &cfg, KernelLaunch &L
         if (v1 <= v0 || v1 - v0 > a.group_size || a.group_ref[u] < v0 || a.group_ref[u] >= v1)
             return cudaErrorInvalidValue;
     }
-    const int smem = static_cast<int>(sizeof(int32_t)) * march_table_entries(a.vol.n);
+    const int smem = static_cast<int>(sizeof(int32_t)) * staged_entries(a.vol.n);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
