@@ -1556,12 +1556,9 @@ __device__ __forceinline__ long long uniform(long long x)
 //
 // The views sit in device memory, so their constants would be loaded into every lane's
 // registers; the ones the march uses in each step are made warp-uniform, which
-// frees 16 registers, and the capped kernel (MINB = 3) then fits in 64 without
-// spills: 32 warps per SM instead of 24.  256 views of a 384^3 x 32 float32 series: 19.49 ->
-// 18.99 ms (64 registers without it spill: 22.8).  The kernel is bound by what L2
-// delivers: with 2 and 4 times the gathers in flight (asynchronous copies into shared memory) it ran no faster.
-template <int STORE, int H, int MINB, bool PAIRED>
-__global__ void __maxnreg__(MINB == 3 ? 64 : 128) region_kernel(const __grid_constant__ RegionArgs a)
+// frees 16 registers.  CAP: the register cap (select_region says which, and why).
+template <int STORE, int H, int CAP, bool PAIRED>
+__global__ void __maxnreg__(CAP) region_kernel(const __grid_constant__ RegionArgs a)
 {
     extern __shared__ int32_t s_tab[];
     const int lane = threadIdx.x & 31;
@@ -1686,33 +1683,40 @@ void *select_kernel(int store, int depth, int capped, int paired)
     return nullptr;
 }
 
-// float32 stages of one cell whatever the depth: that march is bound by L2, and more
-// cells in flight only take registers (see region_kernel).  bfloat16/float16 stages of
-// two: 96 views of 192^2 of 256^3 x 16 1.90 -> 1.64 ms.
-template <int STORE, int MINB, bool PAIRED>
-void *select_region_depth(int depth)
+// The region march waits for its gathers.  Regions of 64 cells and more: what is in flight
+// counts, so stages of `depth` cells and 80 registers, whatever the cap asked for.  Smaller
+// regions: rays of a few dozen cells, where warps count more: 64 registers (80 without the
+// cap), and stages of one cell for float32, which two would spill.
+// Measured (us; stages x registers, two at 80 / one at 64), region 64: 61 views of 192 x 64 of
+// 305^3 x 13 float32 1598 / 1911, 100 views of 128^2 of 320^3 x 16 3322 / 3823, 116 of
+// 98 x 122 of 187^3 x 22 (8-cell bricks) 964 / 1068, 256 of 256^2
+// of 384^3 x 32 (8-cell bricks) 19441 / 19402; region 32: 120
+// views of 224^2 of 320^3 x 12 5703 / 5328.  Stages of one at 80 / 64 registers:
+// 305^3 1645 / 1914.  bfloat16/float16, unpaired, two at 80 / 64 (8 bytes spilled), region
+// 64: 100 views of 100^2 of 300^3 x 16 1196 / 1399; region 32: 1341 / 1171.  Paired records fit
+// in 64 without spills.
+template <int STORE, bool PAIRED>
+void *select_region_stage(int depth, int capped, int region)
 {
-    switch (depth) {
-    case 1: return reinterpret_cast<void *>(&region_kernel<STORE, 1, MINB, PAIRED>);
-    case 2: return reinterpret_cast<void *>(&region_kernel<STORE, STORE == GBD_STORE_F32 ? 1 : 2, MINB, PAIRED>);
-    default: return nullptr;
-    }
+    constexpr bool kF32 = STORE == GBD_STORE_F32;
+    const bool wide = region >= 64 && (kF32 || !PAIRED);
+    const bool two = depth == 2 && (!kF32 || wide);
+    if (depth != 1 && depth != 2) return nullptr;
+    if (capped && !(wide && (kF32 || two)))
+        return two ? reinterpret_cast<void *>(&region_kernel<STORE, kF32 ? 1 : 2, 64, PAIRED>)
+                   : reinterpret_cast<void *>(&region_kernel<STORE, 1, 64, PAIRED>);
+    return two ? reinterpret_cast<void *>(&region_kernel<STORE, 2, 80, PAIRED>)
+               : reinterpret_cast<void *>(&region_kernel<STORE, 1, 80, PAIRED>);
 }
 
-void *select_region(int store, int depth, int capped, int paired)
+void *select_region(int store, int depth, int capped, int paired, int region)
 {
-    if (store == GBD_STORE_F32) {
-        if (paired) return capped ? select_region_depth<GBD_STORE_F32, 3, true>(depth)
-                                  : select_region_depth<GBD_STORE_F32, 1, true>(depth);
-        return capped ? select_region_depth<GBD_STORE_F32, 3, false>(depth)
-                      : select_region_depth<GBD_STORE_F32, 1, false>(depth);
-    }
-    if (store == GBD_STORE_BF16_F16U) {
-        if (paired) return capped ? select_region_depth<GBD_STORE_BF16_F16U, 3, true>(depth)
-                                  : select_region_depth<GBD_STORE_BF16_F16U, 1, true>(depth);
-        return capped ? select_region_depth<GBD_STORE_BF16_F16U, 3, false>(depth)
-                      : select_region_depth<GBD_STORE_BF16_F16U, 1, false>(depth);
-    }
+    if (store == GBD_STORE_F32)
+        return paired ? select_region_stage<GBD_STORE_F32, true>(depth, capped, region)
+                      : select_region_stage<GBD_STORE_F32, false>(depth, capped, region);
+    if (store == GBD_STORE_BF16_F16U)
+        return paired ? select_region_stage<GBD_STORE_BF16_F16U, true>(depth, capped, region)
+                      : select_region_stage<GBD_STORE_BF16_F16U, false>(depth, capped, region);
     return nullptr;
 }
 
@@ -1805,7 +1809,7 @@ cudaError_t launch_screen(const RegionArgs &a, cudaStream_t stream)
 
 cudaError_t launch_region(const RegionArgs &a, const LaunchCfg &cfg, cudaStream_t stream)
 {
-    void *k = select_region(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired);
+    void *k = select_region(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired, a.region);
     const long long regions = static_cast<long long>(a.nreg[0]) * a.nreg[1] * a.nreg[2];
     if (!k || a.n_views < 1 || a.n_views > 65535 || regions < 1 || regions > 65535 || a.ctas_per_view < 1 ||
         a.rays_per_cta != 32 * cfg.cta_warps || !a.image || !a.region_order)
