@@ -462,12 +462,16 @@ void group_views(MarchArgs &a, int gmax)
 
 int launch_units(const MarchArgs &a) { return a.n_groups > 0 ? a.n_groups : a.n_views; }
 
-const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk)
+const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk, cudaStream_t stream)
 {
     const std::array<int, 4> key{width, height, pk.step_x, pk.step_y};
     auto it = ctx.block_orders.find(key);
     if (it != ctx.block_orders.end()) return it->second;
     if (ctx.block_orders.size() >= 64) return nullptr;  // bounded: further geometries keep row order
+    // no allocation and no wait while the caller captures its stream: both would end the capture
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) cudaGetLastError();
+    if (status != cudaStreamCaptureStatusNone) return nullptr;
     std::vector<int> order(static_cast<size_t>(pk.blocks));
     std::vector<double> d2(order.size());
     for (int t = 0; t < pk.blocks; ++t) {
@@ -795,7 +799,7 @@ int render_direct(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, c
         fill_args(*a, vol, hv.data(), n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, cfg,
                   ctx.err_word);
         group_views(*a, cfg.group);
-        if (launch_units(*a) == 1) a->block_order = block_order(ctx, spec.width, spec.height, a->pk);
+        if (launch_units(*a) == 1) a->block_order = block_order(ctx, spec.width, spec.height, a->pk, st);
         e = launch_march(*a, cfg, st);
     }
     if (e == cudaSuccess && spec.out_on_host)
@@ -880,7 +884,7 @@ static cudaError_t chunk_params(Ctx &ctx, const Volume &vol, const GraphKey &key
     float *dev_out = spec.out_on_host ? reinterpret_cast<float *>(g.d_scratch) : spec.out;
     fill_args(a, vol, hv, key.n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, key.cfg, ctx.err_word);
     group_views(a, key.cfg.group);
-    if (launch_units(a) == 1) a.block_order = block_order(ctx, spec.width, spec.height, a.pk);
+    if (launch_units(a) == 1) a.block_order = block_order(ctx, spec.width, spec.height, a.pk, ctx.load_stream);
     KernelLaunch L;
     cudaError_t e = plan_march(a, key.cfg, L);
     if (e != cudaSuccess) return e;
@@ -1493,7 +1497,7 @@ int gbd_render_vector(gbd_ctx *ctx, gbd_volume vid, const gbd_view *views, int32
         a->chan = vol->chan;
         a->chan_comp_stride = vol->chan_stride * vol->grid.n_epochs;
         a->chan_cell_stride = vol->chan_stride;
-        if (launch_units(*a) == 1) a->block_order = block_order(*ctx, spec->width, spec->height, a->pk);
+        if (launch_units(*a) == 1) a->block_order = block_order(*ctx, spec->width, spec->height, a->pk, st);
         e = launch_vector(*a, vol->n_chan, cfg, st);
         ++launches;
     }

@@ -141,9 +141,9 @@ void group_views(MarchArgs &a, int gmax);
 // The order in which the CTAs of a launch of one view or time group take its
 // blocks: by distance of the block from the image centre, nearest first (the longest
 // rays of a centred box first, so the launch ends on short ones).  A device table cached
-// in the context for up to 64 image geometries; NULL (row order) beyond them or
-// if it cannot be made.  Launches of several views run view after view in row order.
-const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk);
+// in the context for up to 64 image geometries; NULL (row order) beyond them,
+// if it cannot be made, or on its first use while `stream` is captured.  Launches of several views run view after view in row order.
+const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk, cudaStream_t stream);
 // Views, or time groups when grouped, of a filled launch.
 int launch_units(const MarchArgs &a);
 bool build_layout(const int n[3], int B, int S, std::vector<int32_t> &tab, long long &epoch_stride, int morton_cells);
