@@ -320,8 +320,6 @@ int check_spec(const gbd_image_spec *s)
 
 int march_chunks(int n) { return (n + kViewsPerLaunch - 1) / kViewsPerLaunch; }
 
-// Launch arguments of chunk c of a batch of n views: views c K .. c K + K - 1
-// (K = kViewsPerLaunch) and their images.
 // Two views have the same rays when every per-view constant but the epoch
 // coordinate at the image plane, the window and the prefactor agrees: the
 // same image plane, direction, grid frame, epoch rate per face and boost.
@@ -337,29 +335,56 @@ static bool same_rays(const ViewDev &x, const ViewDev &y)
            x.flags == y.flags;
 }
 
-// Which units a launch takes side by side, block by block: consecutive views (or
-// time groups, by their references) with the same rays whose observer times lie less
-// than two snapshots from one to the next.  At every cell such neighbours read a common
-// snapshot, which the second then finds in a cache; further apart or along other rays
-// they share no record.  18 float32 images of 512^2 of a 256^3 x 16 series, one after
-// the other / side by side: lone marches 860 / 833 us, groups of three 583 / 549.
+// Which units (views, or time groups, by their references) a launch takes side by side,
+// block by block, the blocks of lone marches centre of the image first.
+//  * Consecutive units with the same rays whose observer times lie less than two snapshots
+//    from one to the next: at every cell such neighbours read a common snapshot, which
+//    the second then finds in a cache; further apart they share no record.  18 float32
+//    images of 512^2 of a 256^3 x 16 series, one after the other / side by side: lone marches
+//    860 / 833 us, groups of three 583 / 549.
+//  * Lone marches along different rays, as many at a time as have about kRunPixels pixels:
+//    view after view, the chip works on rays of one length, many and short at an image's
+//    edges and few and long at its end; side by side the long rays come first for all of
+//    them, and the views read the same cells at about the same time.  One after the other /
+//    so: 12 views of 200^2 of 128^3 x 8 float32 141 / 129 us, 100 of 256^2 of 256^3 x 16
+//    9183 / 7979 (bfloat16/float16 4593 / 4004), 24 of 256^2 of 320^3 x 16 3983 / 3772, three channels
+//    of 4 of 192^2 of 160^3 x 6 327 / 271.  Larger images drift apart: 24 of 384^2 of 256^3 x 16
+//    2491 / 2532, with all of them side by side 2592.
+constexpr long long kRunPixels = 1 << 20;
 static void set_runs(MarchArgs &a)
 {
     const int units = a.n_groups > 0 ? a.n_groups : a.n_views;
     auto view = [&](int u) -> const ViewDev & { return a.views[a.n_groups > 0 ? a.group_ref[u] : u]; };
-    for (int u = 0; u < units;) {
-        int e = u + 1;
-        while (e < units && same_rays(view(u), view(e)) &&
-               std::llabs(view(e).u_obs - view(e - 1).u_obs) < (2LL << 32))
-            ++e;
+    // unit u + 1 exists and has unit u's rays
+    auto joined = [&](int u) { return u + 1 < units && same_rays(view(u), view(u + 1)); };
+    auto apart = [&](int u) { return std::llabs(view(u + 1).u_obs - view(u).u_obs); };
+    auto run = [&](int u, int e) {
         for (int k = u; k < e; ++k) {
             a.run_first[k] = static_cast<short>(u);
             a.run_len[k] = static_cast<short>(e - u);
+        }
+    };
+    a.near_units = 0;
+    for (int u = 0; u < units;) {
+        int e = u + 1;
+        if (joined(u) || a.n_groups > 0) {
+            while (joined(e - 1) && apart(e - 1) < (2LL << 32)) {
+                a.near_units += apart(e - 1) < (1LL << 32) ? 1 : 0;
+                ++e;
+            }
+            run(u, e);
+        } else {
+            while (e < units && !joined(e - 1) && !joined(e)) ++e;
+            const int most = static_cast<int>(std::max(1LL, kRunPixels / (static_cast<long long>(a.width) * a.height)));
+            const int parts = (e - u + most - 1) / most;
+            for (int k = 0; k < parts; ++k) run(u + (e - u) * k / parts, u + (e - u) * (k + 1) / parts);
         }
         u = e;
     }
 }
 
+// Launch arguments of chunk c of a batch of n views: views c K .. c K + K - 1
+// (K = kViewsPerLaunch) and their images.
 void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c, const gbd_image_spec &s,
                float *out, uint32_t *samples, const LaunchCfg &cfg, int *err_word)
 {
@@ -460,7 +485,7 @@ void group_views(MarchArgs &a, int gmax)
     set_runs(a);
 }
 
-int launch_units(const MarchArgs &a) { return a.n_groups > 0 ? a.n_groups : a.n_views; }
+bool takes_order(const MarchArgs &a) { return a.n_groups <= 1 && a.near_units == 0; }
 
 const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk, cudaStream_t stream)
 {
@@ -799,7 +824,7 @@ int render_direct(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, c
         fill_args(*a, vol, hv.data(), n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, cfg,
                   ctx.err_word);
         group_views(*a, cfg.group);
-        if (launch_units(*a) == 1) a->block_order = block_order(ctx, spec.width, spec.height, a->pk, st);
+        if (takes_order(*a)) a->block_order = block_order(ctx, spec.width, spec.height, a->pk, st);
         e = launch_march(*a, cfg, st);
     }
     if (e == cudaSuccess && spec.out_on_host)
@@ -884,7 +909,7 @@ static cudaError_t chunk_params(Ctx &ctx, const Volume &vol, const GraphKey &key
     float *dev_out = spec.out_on_host ? reinterpret_cast<float *>(g.d_scratch) : spec.out;
     fill_args(a, vol, hv, key.n, c, spec, dev_out, spec.out_on_host ? nullptr : spec.samples, key.cfg, ctx.err_word);
     group_views(a, key.cfg.group);
-    if (launch_units(a) == 1) a.block_order = block_order(ctx, spec.width, spec.height, a.pk, ctx.load_stream);
+    if (takes_order(a)) a.block_order = block_order(ctx, spec.width, spec.height, a.pk, ctx.load_stream);
     KernelLaunch L;
     cudaError_t e = plan_march(a, key.cfg, L);
     if (e != cudaSuccess) return e;
@@ -1497,7 +1522,7 @@ int gbd_render_vector(gbd_ctx *ctx, gbd_volume vid, const gbd_view *views, int32
         a->chan = vol->chan;
         a->chan_comp_stride = vol->chan_stride * vol->grid.n_epochs;
         a->chan_cell_stride = vol->chan_stride;
-        if (launch_units(*a) == 1) a->block_order = block_order(*ctx, spec->width, spec->height, a->pk, st);
+        a->block_order = block_order(*ctx, spec->width, spec->height, a->pk, st);
         e = launch_vector(*a, vol->n_chan, cfg, st);
         ++launches;
     }

@@ -137,7 +137,7 @@ struct MarchArgs {
     int n_views;              // views in this launch, 1 .. kViewsPerLaunch
     int width, height;
     PacketGrid pk;            // how the CTAs and warps cover an image
-    const int *block_order;   // CTA of an image -> its block (centre of the image first), or NULL: in row order
+    const int *block_order;   // n-th block that a launch takes of an image (centre first), or NULL: in row order
     int n_groups;             // 0: every view marched on its own; else time groups of consecutive views
     int group_size;           // time groups: the kernel's member limit (4 or kGroupMax)
     int group_snaps;          // and its snapshots per cell (kGroupSnapsMin or kGroupSnapsMax)
@@ -148,6 +148,7 @@ struct MarchArgs {
     // units (views, or time groups) that the launch takes side by side: unit u is in the
     // run of run_len[u] units from run_first[u]
     short run_first[kViewsPerLaunch], run_len[kViewsPerLaunch];
+    int near_units;           // units within a snapshot of the one before, along the same rays (host only)
     int accumulate;           // add to out (and samples) instead of storing
     float *out;               // n_views * width * height floats
     uint32_t *samples;        // optional, same shape

@@ -1261,7 +1261,7 @@ __global__ void __maxnreg__(96) vector_kernel(const __grid_constant__ MarchArgs 
 {
     extern __shared__ int32_t s_mem[];
     int32_t *s_tab = s_mem + kSpanEntries;
-    const BlockWork w = block_work<false>(a);
+    const BlockWork w = block_work<true>(a);
     const ViewDev &V = a.views[w.unit];
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);

@@ -138,14 +138,15 @@ void fill_args(MarchArgs &a, const Volume &vol, const ViewDev *hv, int n, int c,
                float *out, uint32_t *samples, const LaunchCfg &cfg, int *err_word);
 // Time groups of a filled launch (batched renders; see MarchArgs).
 void group_views(MarchArgs &a, int gmax);
-// The order in which the CTAs of a launch of one view or time group take its
-// blocks: by distance of the block from the image centre, nearest first (the longest
-// rays of a centred box first, so the launch ends on short ones).  A device table cached
-// in the context for up to 64 image geometries; NULL (row order) beyond them,
-// if it cannot be made, or on its first use while `stream` is captured.  Launches of several views run view after view in row order.
+// The order in which a launch takes an image's blocks: by distance of the block from the
+// image centre, nearest first (the longest rays of a centred box first, so the launch
+// ends on short ones).  A device table cached in the context for up to 64 image
+// geometries; NULL (row order) beyond them, if it cannot be made, or on its first use while `stream` is captured.
 const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk, cudaStream_t stream);
-// Views, or time groups when grouped, of a filled launch.
-int launch_units(const MarchArgs &a);
+// The launches that use it: all but those of several time groups or of views within a
+// snapshot of each other along the same rays, whose neighbouring CTAs share more on
+// neighbouring blocks (24 views 0.1 snapshots apart, paired float32: 1025 us, in this order 1073).
+bool takes_order(const MarchArgs &a);
 bool build_layout(const int n[3], int B, int S, std::vector<int32_t> &tab, long long &epoch_stride, int morton_cells);
 void destroy_graph_cache(GraphCache *g);
 

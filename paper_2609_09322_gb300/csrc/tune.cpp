@@ -89,7 +89,7 @@ int time_config(Ctx &ctx, const Volume &vol, const std::vector<ViewDev> &hv, con
         for (int c = 0; c < chunks && e == cudaSuccess && slots == 0; ++c) {
             fill_args(*args, vol, hv.data(), n, c, spec, spec.out, nullptr, cfg, ctx.err_word);
             group_views(*args, cfg.group);
-            if (launch_units(*args) == 1) args->block_order = block_order(ctx, spec.width, spec.height, args->pk, st);
+            if (takes_order(*args)) args->block_order = block_order(ctx, spec.width, spec.height, args->pk, st);
             e = launch_march(*args, cfg, st);
         }
         if (e == cudaSuccess) e = cudaEventRecord(b, st);

@@ -50,3 +50,27 @@ def test_region_kernels_agree(ctx, n, region, store, paired):
                                       what=f"{n} region {region} view {k}")
                 assert torch.equal(img, want), (depth, regcap, warps)
     ctx.unload(vol)
+
+
+@pytest.mark.parametrize("store", ["f32", "bf16"])
+@pytest.mark.parametrize("size", [(64, 64), (23, 41), (700, 400)])
+def test_views_side_by_side_equal_single_renders(ctx, store, size):
+    """Views along different rays and along the same ones, in runs of every kind: a batch's
+    images and a vector render's are the single renders' bit for bit."""
+    w, h = size
+    grid, j, beta = even_grid(9, (21, 15, 18), 4)
+    vol = ctx.load_snapshots(grid, j, beta, store=store)
+    ctx.load_channels(vol, np.stack([2.0 * j, j, -j]))
+    fov = 1.8 * float(np.max(grid.extent))
+    views = [gen.view_from_direction(grid, -d, size=w, fov=fov, height=h, c=1.3).with_(fov_v=fov, t_obs=3.0)
+             for d in gen.fibonacci_directions(9)]
+    series = [views[2].with_(t_obs=3.0 + 1.1 * k) for k in range(3)]
+    batch = views[:5] + series + views[5:] + [series[0], views[0].with_(t_obs=9.5), views[0]]
+    singles = [ctx.render(vol, v) for v in batch]
+    got = ctx.render_batch(vol, batch, launch={"group": 1})
+    vec = ctx.render_vector(vol, batch)
+    one = torch.stack([ctx.render_vector(vol, [v])[0] for v in batch])
+    torch.cuda.synchronize()
+    assert torch.equal(got, torch.stack(singles)) and torch.equal(vec, one)
+    assert float(got.max()) > 0
+    ctx.unload(vol)

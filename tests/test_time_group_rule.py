@@ -113,3 +113,87 @@ def test_groups_are_the_fewest_and_close(rule, m, gmax):
 
 def test_one_late_view_leaves_the_others_grouped(rule):
     assert [len(x) - 2 for x in rule([(16, 4, t) for t in SERIES[:4]])] == [6, 7, 7, 7]
+
+
+RUNS_PROGRAM = r"""
+#include <cstdio>
+#include <cstring>
+#include <memory>
+#include <vector>
+#include "runtime.h"
+int main()
+{
+    int w, h, n;
+    while (std::scanf("%d %d %d", &w, &h, &n) == 3) {
+        std::vector<gbd::ViewDev> hv(n);
+        std::memset(hv.data(), 0, sizeof(gbd::ViewDev) * n);
+        for (int v = 0; v < n; ++v) {
+            int dir;
+            double u;
+            if (std::scanf("%d %lf", &dir, &u) != 2) return 1;
+            hv[v].g0[0] = dir;
+            hv[v].u_obs = static_cast<long long>(u * 4294967296.0);
+        }
+        gbd::Volume vol;
+        vol.grid.n[0] = vol.grid.n[1] = vol.grid.n[2] = 4;
+        vol.grid.n_epochs = 4;
+        gbd_image_spec s{};
+        s.width = w;
+        s.height = h;
+        auto a = std::make_unique<gbd::MarchArgs>();
+        gbd::fill_args(*a, vol, hv.data(), n, 0, s, nullptr, nullptr, gbd::LaunchCfg{8, 4, 4, 2, 1, 1, 0, 4}, nullptr);
+        std::printf("%d", a->near_units);
+        for (int v = 0; v < n; ++v) std::printf(" %d:%d", a->run_first[v], a->run_len[v]);
+        std::printf("\n");
+    }
+    std::fflush(stdout);
+    std::_Exit(0);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def runs(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    gbdart.load_library()
+    d = tmp_path_factory.mktemp("runs")
+    (d / "runs.cpp").write_text(RUNS_PROGRAM.replace("#include <cstdio>", "#include <cstdio>\n#include <cstdlib>"))
+    subprocess.run([cxx, "-std=c++17", "-I", build.CSRC, "-I", os.path.join(CUDA, "include"), str(d / "runs.cpp"),
+                    build.lib_path(), "-Wl,-rpath," + build.BUILD, "-Wl,--allow-shlib-undefined", "-o",
+                    str(d / "runs")], check=True, capture_output=True)
+
+    def run(w, h, views):
+        text = f"{w} {h} {len(views)} " + " ".join(f"{d} {u}" for d, u in views) + "\n"
+        env = dict(os.environ)
+        env["LD_LIBRARY_PATH"] = os.path.join(CUDA, "lib64") + ":" + env.get("LD_LIBRARY_PATH", "")
+        out = subprocess.run([str(d / "runs")], input=text, check=True, capture_output=True, text=True, env=env).stdout
+        near, *pairs = out.split()
+        first = [tuple(int(x) for x in p.split(":")) for p in pairs]
+        # runs are whole: every unit names the run it is in
+        at = 0
+        lens = []
+        while at < len(views):
+            f, k = first[at]
+            assert f == at and k >= 1 and first[at:at + k] == [(f, k)] * k
+            lens.append(k)
+            at += k
+        return int(near), lens
+
+    return run
+
+
+def test_which_views_go_side_by_side(runs):
+    dirs = [(k, 1.0) for k in range(24)]
+    assert runs(256, 256, dirs[:16]) == (0, [16])                       # 2^20 pixels at a time
+    assert runs(256, 256, dirs) == (0, [12, 12])                        # in equal parts
+    assert runs(1024, 1024, dirs[:3]) == (0, [1, 1, 1])
+    assert runs(16384, 16384, dirs[:2]) == (0, [1, 1])
+    assert runs(1, 1, [(k, 0.0) for k in range(128)]) == (0, [128])
+    same = [(0, 0.5 * k) for k in range(9)]
+    assert runs(512, 512, same) == (8, [9])                             # whatever their size
+    assert runs(512, 512, [(0, 1.5 * k) for k in range(5)]) == (0, [5])
+    assert runs(512, 512, [(0, 2.0 * k) for k in range(5)]) == (0, [1] * 5)
+    # two other directions, a series, and one more direction
+    assert runs(64, 64, [(1, 0.0), (2, 0.0)] + same + [(3, 0.0)]) == (8, [2, 9, 1])
