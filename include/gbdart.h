@@ -165,10 +165,12 @@ typedef struct {
     int32_t packet_w, packet_h;  /* pixels of one warp packet: 8x4, 4x8, 16x2, 32x1 */
     int32_t cta_warps;           /* warps per CTA: 1, 2, 4 or 8                     */
     int32_t depth;               /* cells gathered ahead per lane, while as many are
-                                    evaluated: 1, 2 or 4 (4 runs as 2)             */
+                                    evaluated: 1 = one, 4 = two, 2 = whichever suits
+                                    the launch (the images are the same)         */
     int32_t persistent;          /* accepted, 0 or 1, without effect: every launch
-                                    is one packet per warp, view after view      */
-    int32_t regcap;              /* 1 = kernel built for at most 80 registers/thread */
+                                    is one packet per warp                       */
+    int32_t regcap;              /* 1 = kernel built for at most 80 registers/thread
+                                    (region schedule: 64 or 80)                  */
     int32_t region;              /* batches: 0 = march every ray whole; 16, 32, 64
                                     or 128 = region schedule: march all views' rays
                                     region by region (edge^3 cells, while the region

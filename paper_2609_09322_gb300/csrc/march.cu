@@ -1833,13 +1833,53 @@ cudaError_t launch_reduce(const ReduceArgs &a, cudaStream_t stream)
                             0, stream);
 }
 
+// Cells of a stage at depth 2, the default.  Unpaired float32 stages of two cells take 80
+// registers (24 warps per SM), of one 64 (32 warps): two hide the latency of DRAM, one does
+// more work where L1 and L2 deliver.  One cell where the records that a launch reads come
+// from the caches:
+//  * kDenseRays rays and more through a cell: its record is read again at once;
+//  * the snapshots around a time (or the only one) fit in L2 with room to spare;
+//  * one snapshot: half the loads of a sample;
+//  * half of the views within a snapshot of the one before, along the same rays.
+// And only in launches that fill 32 warps per SM about one and a half times: with fewer, each
+// ray's own latency counts.  Two cells / one, us: dense: 1024^2 of 128^3 x 8 324 / 270, six
+// views of 512^2 of 200^3 x 8 (3.3 rays) 520 / 460, 1024^2 of 384^3 x 6 (3.6) 1009 / 1023, 512^2 of 256^3
+// x 8 (2.0) 236 / 282; L2: 12 of 256^2 of 160^3 x 8 (131 MB) 231 / 220, 6 of 300^2 of 200^3 x 12 (256 MB)
+// 279 / 314; one snapshot: 1024^2 of 512^3 741 / 639; series: 18 of 512^2 of 256^3 x 16, marched alone,
+// 942 / 826; few warps: 24 of 100^2 of 160^3 x 8 (7500) 176 / 198, 512^2 of 100^3 x 8 (8192) 84 / 76.
+// Paired records (one pair for a sample) and bfloat16/float16 take two: 24 of 384^2 of 256^3 x 16
+// 2290 / 2337 paired, 1627 / 1716 in bfloat16/float16.
+constexpr double kDenseRays = 3.2;
+constexpr long long kCachedBytes = 128LL << 20;
+constexpr long long kFullWarps = 8000;
+int stage_cells(const MarchArgs &a)
+{
+    if (a.vol.store != GBD_STORE_F32 || a.vol.paired) return 2;
+    const long long warps = static_cast<long long>(a.n_views) * a.pk.blocks * (a.pk.step_x * a.pk.step_y / 32);
+    if (warps < kFullWarps) return 2;
+    const long long cells = static_cast<long long>(a.vol.n[0]) * a.vol.n[1] * a.vol.n[2];
+    if (a.vol.M == 1 || cells * 2 * 16 <= kCachedBytes || 2 * a.near_units >= a.n_views) return 1;
+    // rays through a unit cell: its projected area over a pixel's, both times |a|
+    const ViewDev &V = a.views[0];
+    double u[3], v[3], d[3];
+    for (int i = 0; i < 3; ++i) {
+        u[i] = static_cast<double>(V.gu[i]) * 0x1p-40;
+        v[i] = static_cast<double>(V.gv[i]) * 0x1p-40;
+        d[i] = V.a_hi[i];
+    }
+    const double pixel = d[0] * (u[1] * v[2] - u[2] * v[1]) + d[1] * (u[2] * v[0] - u[0] * v[2]) +
+                         d[2] * (u[0] * v[1] - u[1] * v[0]);
+    return d[0] + d[1] + d[2] >= kDenseRays * (pixel < 0.0 ? -pixel : pixel) ? 1 : 2;
+}
+
 cudaError_t plan_march(const MarchArgs &a, const LaunchCfg &cfg, KernelLaunch &L)
 {
     // n_groups > 0: time groups, one image's blocks of CTAs per group; else per view
     const bool grouped = a.n_groups > 0;
     void *k = grouped ? select_group(a.vol.store, a.group_size, cfg.depth, a.group_snaps,
                                      march_table_entries(a.vol.n) > kCopiesMax * 32 * cfg.cta_warps)
-                      : select_kernel(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired);
+                      : select_kernel(a.vol.store, cfg.depth == 2 ? stage_cells(a) : cfg.depth, cfg.regcap,
+                                      a.vol.paired);
     if (!k || a.n_views < 1 || a.n_views > kViewsPerLaunch) return cudaErrorInvalidValue;
     if (grouped && (a.n_groups > a.n_views || a.group_first[0] != 0 || a.group_first[a.n_groups] != a.n_views))
         return cudaErrorInvalidValue;

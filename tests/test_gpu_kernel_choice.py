@@ -74,3 +74,25 @@ def test_views_side_by_side_equal_single_renders(ctx, store, size):
     assert torch.equal(got, torch.stack(singles)) and torch.equal(vec, one)
     assert float(got.max()) > 0
     ctx.unload(vol)
+
+
+# 8000 warps of 8x4 pixels, one snapshot or three, dense rays or not, lone series
+@pytest.mark.parametrize("w,h,views", [(512, 499, 1), (512, 500, 1), (512, 516, 1), (300, 290, 3)])
+@pytest.mark.parametrize("m,paired", [(1, False), (3, False), (3, True)])
+def test_stage_depths_agree(ctx, w, h, views, m, paired):
+    grid, j, beta = even_grid(10 + m, (26, 33, 19), m)
+    vol = ctx.load_snapshots(grid, j, beta, paired=paired)
+    fov = 1.8 * float(np.max(grid.extent))
+    base = gen.view_from_angles(grid, 37.0, 205.0, size=w, fov=fov, c=20.0).with_(height=h, fov_v=fov, t_obs=2.0)
+    series = [base.with_(t_obs=2.0 + 0.3 * k) for k in range(views)]
+    want = ctx.render_batch(vol, series, launch={"depth": 1, "group": 1})
+    want = want.clone()
+    assert float(want.max()) > 0
+    for depth in (2, 4):
+        for regcap in (0, 1):
+            got = ctx.render_batch(vol, series, launch={"depth": depth, "group": 1, "regcap": regcap})
+            assert torch.equal(got, want), (depth, regcap)
+    px = np.random.default_rng(1).integers(0, (w, h), size=(40, 2))
+    assert_parity(want[0].cpu().numpy()[px[:, 1], px[:, 0]], oracle.render_pixels(grid, j, beta, series[0], px),
+                  what=f"{w}x{h} M {m}")
+    ctx.unload(vol)
