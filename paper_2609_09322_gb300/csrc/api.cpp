@@ -744,6 +744,9 @@ cudaError_t enqueue_regions(Ctx &ctx, const Volume &vol, const std::vector<ViewD
     a.packet_w = cfg.packet_w;
     a.packet_h = cfg.packet_h;
     a.region = cfg.region;
+    double rays = 0.0;
+    for (const ViewDev &V : hv) rays += rays_per_cell(V);
+    a.rays_per_cell = static_cast<float>(rays / n);
     for (int i = 0; i < 3; ++i) a.nreg[i] = P.nreg[i];
     a.partial = partial;
     a.slot_stride = slot_stride;

@@ -90,6 +90,21 @@ struct ViewDev {
     uint32_t flags;    // GBD_BEAMING | GBD_LOOKBACK | kFlagMirror0 << axis
 };
 
+// Rays of a view through a unit cell: the cell's projected area over a pixel's (both times
+// the direction's length), on the host.
+inline double rays_per_cell(const ViewDev &V)
+{
+    double u[3], v[3], d[3];
+    for (int i = 0; i < 3; ++i) {
+        u[i] = static_cast<double>(V.gu[i]) * 0x1p-40;
+        v[i] = static_cast<double>(V.gv[i]) * 0x1p-40;
+        d[i] = V.a_hi[i];
+    }
+    const double pixel = d[0] * (u[1] * v[2] - u[2] * v[1]) + d[1] * (u[2] * v[0] - u[0] * v[2]) +
+                         d[2] * (u[0] * v[1] - u[1] * v[0]);
+    return (d[0] + d[1] + d[2]) / (pixel < 0.0 ? -pixel : pixel);
+}
+
 // Views per march launch.  The views travel in the kernel's parameter space
 // (up to 32 KB on sm_70 and later with CUDA 12.1+), and each CTA works on one
 // view, so every per-view constant is uniform across the CTA and the compiler
@@ -190,6 +205,7 @@ struct RegionArgs {
     int width, height;
     int packet_w, packet_h;
     int region;               // region edge in cells
+    float rays_per_cell;      // mean of the views (host only: which kernel)
     int nreg[3];              // regions per axis
     float *partial;           // slot s of batch image b at partial + s * slot_stride + b * width * height
     long long slot_stride;    // floats per slot

@@ -1683,40 +1683,49 @@ void *select_kernel(int store, int depth, int capped, int paired)
     return nullptr;
 }
 
-// The region march waits for its gathers.  Regions of 64 cells and more: what is in flight
-// counts, so stages of `depth` cells and 80 registers, whatever the cap asked for.  Smaller
-// regions: rays of a few dozen cells, where warps count more: 64 registers (80 without the
-// cap), and stages of one cell for float32, which two would spill.
-// Measured (us; stages x registers, two at 80 / one at 64), region 64: 61 views of 192 x 64 of
-// 305^3 x 13 float32 1598 / 1911, 100 views of 128^2 of 320^3 x 16 3322 / 3823, 116 of
-// 98 x 122 of 187^3 x 22 (8-cell bricks) 964 / 1068, 256 of 256^2
-// of 384^3 x 32 (8-cell bricks) 19441 / 19402; region 32: 120
-// views of 224^2 of 320^3 x 12 5703 / 5328.  Stages of one at 80 / 64 registers:
-// 305^3 1645 / 1914.  bfloat16/float16, unpaired, two at 80 / 64 (8 bytes spilled), region
-// 64: 100 views of 100^2 of 300^3 x 16 1196 / 1399; region 32: 1341 / 1171.  Paired records fit
-// in 64 without spills.
-template <int STORE, bool PAIRED>
-void *select_region_stage(int depth, int capped, int region)
+// The region march waits for its gathers.  Where few rays cross a region (64 cells and more,
+// few rays through a cell), what is in flight counts: stages of `depth` cells and 80 registers,
+// whatever the cap asked for.  Elsewhere warps count more: 64 registers, and for
+// float32 (which two cells would spill; 80 without the cap) stages of one cell.
+// Paired bfloat16/float16 records fit two cells in 64.
+// Measured, two cells at 80 registers / the others (us), regions of 64. float32 (one at 64), by rays
+// through a cell: 1.1: 60 views of 216^2 of 147^3 x 6 729 / 692; 0.4: 224^2 of 250^3 1181 / 1158;
+// 0.35: 64 of 160^2 of 192^3 x 12 850 / 892; 0.2: 256 of 256^2 of 384^3 x 32 (8-cell bricks) 19441 / 19402, 61 of
+// 192 x 64 of 305^3 x 13 1602 / 1913; 0.08: 100 of 128^2 of 320^3 x 16 3331 / 3830; regions of 128, 0.4:
+// 1392 / 1478, of 32, 0.28: 5703 / 5328.  bfloat16/float16, unpaired (two at 64, 8 bytes spilled): 1.1: 158 of
+// 216 x 91 of 147^3 x 6 987 / 917; 0.28: 60 of 224^2 of 300^3 1167 / 1123; 0.055: 100 of 100^2 of 300^3 x 16
+// 1197 / 1400; regions of 128, 0.32: 100 of 200^2 of 250^3 x 16 2382 / 2671; of 32, 0.055: 1341 / 1171.
+bool sparse_regions(int store, int paired, int region, float rays)
 {
-    constexpr bool kF32 = STORE == GBD_STORE_F32;
-    const bool wide = region >= 64 && (kF32 || !PAIRED);
-    const bool two = depth == 2 && (!kF32 || wide);
-    if (depth != 1 && depth != 2) return nullptr;
-    if (capped && !(wide && (kF32 || two)))
-        return two ? reinterpret_cast<void *>(&region_kernel<STORE, kF32 ? 1 : 2, 64, PAIRED>)
-                   : reinterpret_cast<void *>(&region_kernel<STORE, 1, 64, PAIRED>);
-    return two ? reinterpret_cast<void *>(&region_kernel<STORE, 2, 80, PAIRED>)
-               : reinterpret_cast<void *>(&region_kernel<STORE, 1, 80, PAIRED>);
+    if (region < 64) return false;
+    if (store == GBD_STORE_F32) return rays < (region >= 128 ? 0.5f : 0.375f);
+    return !paired && rays < (region >= 128 ? 0.35f : 0.15f);
 }
 
-void *select_region(int store, int depth, int capped, int paired, int region)
+template <bool PAIRED>
+void *select_region_f32(int depth, int capped, bool sparse)
 {
+    if (sparse && depth == 2) return reinterpret_cast<void *>(&region_kernel<GBD_STORE_F32, 2, 80, PAIRED>);
+    return capped && !sparse ? reinterpret_cast<void *>(&region_kernel<GBD_STORE_F32, 1, 64, PAIRED>)
+                             : reinterpret_cast<void *>(&region_kernel<GBD_STORE_F32, 1, 80, PAIRED>);
+}
+
+template <bool PAIRED>
+void *select_region_bf16(int depth)
+{
+    return depth == 2 ? reinterpret_cast<void *>(&region_kernel<GBD_STORE_BF16_F16U, 2, 64, PAIRED>)
+                      : reinterpret_cast<void *>(&region_kernel<GBD_STORE_BF16_F16U, 1, 64, PAIRED>);
+}
+
+void *select_region(int store, int depth, int capped, int paired, bool sparse)
+{
+    if (depth != 1 && depth != 2) return nullptr;
     if (store == GBD_STORE_F32)
-        return paired ? select_region_stage<GBD_STORE_F32, true>(depth, capped, region)
-                      : select_region_stage<GBD_STORE_F32, false>(depth, capped, region);
-    if (store == GBD_STORE_BF16_F16U)
-        return paired ? select_region_stage<GBD_STORE_BF16_F16U, true>(depth, capped, region)
-                      : select_region_stage<GBD_STORE_BF16_F16U, false>(depth, capped, region);
+        return paired ? select_region_f32<true>(depth, capped, sparse) : select_region_f32<false>(depth, capped, sparse);
+    if (store == GBD_STORE_BF16_F16U) {
+        if (sparse && depth == 2) return reinterpret_cast<void *>(&region_kernel<GBD_STORE_BF16_F16U, 2, 80, false>);
+        return paired ? select_region_bf16<true>(depth) : select_region_bf16<false>(depth);
+    }
     return nullptr;
 }
 
@@ -1809,7 +1818,8 @@ cudaError_t launch_screen(const RegionArgs &a, cudaStream_t stream)
 
 cudaError_t launch_region(const RegionArgs &a, const LaunchCfg &cfg, cudaStream_t stream)
 {
-    void *k = select_region(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired, a.region);
+    void *k = select_region(a.vol.store, cfg.depth, cfg.regcap, a.vol.paired,
+                            sparse_regions(a.vol.store, a.vol.paired, a.region, a.rays_per_cell));
     const long long regions = static_cast<long long>(a.nreg[0]) * a.nreg[1] * a.nreg[2];
     if (!k || a.n_views < 1 || a.n_views > 65535 || regions < 1 || regions > 65535 || a.ctas_per_view < 1 ||
         a.rays_per_cta != 32 * cfg.cta_warps || !a.image || !a.region_order)
@@ -1859,17 +1869,7 @@ int stage_cells(const MarchArgs &a)
     if (warps < kFullWarps) return 2;
     const long long cells = static_cast<long long>(a.vol.n[0]) * a.vol.n[1] * a.vol.n[2];
     if (a.vol.M == 1 || cells * 2 * 16 <= kCachedBytes || 2 * a.near_units >= a.n_views) return 1;
-    // rays through a unit cell: its projected area over a pixel's, both times |a|
-    const ViewDev &V = a.views[0];
-    double u[3], v[3], d[3];
-    for (int i = 0; i < 3; ++i) {
-        u[i] = static_cast<double>(V.gu[i]) * 0x1p-40;
-        v[i] = static_cast<double>(V.gv[i]) * 0x1p-40;
-        d[i] = V.a_hi[i];
-    }
-    const double pixel = d[0] * (u[1] * v[2] - u[2] * v[1]) + d[1] * (u[2] * v[0] - u[0] * v[2]) +
-                         d[2] * (u[0] * v[1] - u[1] * v[0]);
-    return d[0] + d[1] + d[2] >= kDenseRays * (pixel < 0.0 ? -pixel : pixel) ? 1 : 2;
+    return rays_per_cell(a.views[0]) >= kDenseRays ? 1 : 2;
 }
 
 cudaError_t plan_march(const MarchArgs &a, const LaunchCfg &cfg, KernelLaunch &L)
