@@ -1657,7 +1657,9 @@ void *select_group_size(int size, int snaps)
 // float32 groups march one cell per iteration whatever the depth, and
 // bfloat16/float16 ones at most two: a cell's S gathers already keep as many
 // loads in flight, and more cells' records would cost more warps than the
-// loads gain.
+// loads gain.  Groups of more than four with five snapshots take one: two spill 108 bytes
+// (8 views of 384^2 of 256^3 x 32 within 2.9 snapshots 311 / 300 us; with three snapshots, 8
+// bytes spilled, within 0.9: 197 / 218).
 // Long tables (spans): one kernel per store, for any group.
 void *select_group(int store, int size, int depth, int snaps, bool spans)
 {
@@ -1667,10 +1669,12 @@ void *select_group(int store, int size, int depth, int snaps, bool spans)
                    ? reinterpret_cast<void *>(&group_kernel<GBD_STORE_F32, 1, kGroupMax, kGroupSnapsMax, true>)
                    : reinterpret_cast<void *>(&group_kernel<GBD_STORE_BF16_F16U, 1, kGroupMax, kGroupSnapsMax, true>);
     if (store == GBD_STORE_F32) return select_group_size<GBD_STORE_F32, 1>(size, snaps);
-    if (store == GBD_STORE_BF16_F16U)
-        return depth == 1 ? select_group_size<GBD_STORE_BF16_F16U, 1>(size, snaps)
-                          : select_group_size<GBD_STORE_BF16_F16U, 2>(size, snaps);
-    return nullptr;
+    if (store != GBD_STORE_BF16_F16U) return nullptr;
+    if (depth == 1 || (size == kGroupMax && snaps == kGroupSnapsMax))
+        return select_group_size<GBD_STORE_BF16_F16U, 1>(size, snaps);
+    if (size == kGroupMax)
+        return reinterpret_cast<void *>(&group_kernel<GBD_STORE_BF16_F16U, 2, kGroupMax, kGroupSnapsMin, false>);
+    return select_group_snaps<GBD_STORE_BF16_F16U, 2, 4>(snaps);
 }
 
 void *select_kernel(int store, int depth, int capped, int paired)
