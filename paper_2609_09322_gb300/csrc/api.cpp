@@ -336,7 +336,7 @@ static bool same_rays(const ViewDev &x, const ViewDev &y)
 }
 
 // Which units (views, or time groups, by their references) a launch takes side by side,
-// block by block, the blocks of lone marches centre of the image first.
+// block by block; the blocks of lone marches along different rays go centre first.
 //  * Consecutive units with the same rays whose observer times lie less than two snapshots
 //    from one to the next: at every cell such neighbours read a common snapshot, which
 //    the second then finds in a cache; further apart they share no record.  18 float32
@@ -381,6 +381,7 @@ static void set_runs(MarchArgs &a)
         }
         u = e;
     }
+    a.rows_from_middle = a.n_groups == 0 && a.near_units == 0;
 }
 
 // Launch arguments of chunk c of a batch of n views: views c K .. c K + K - 1
@@ -485,7 +486,11 @@ void group_views(MarchArgs &a, int gmax)
     set_runs(a);
 }
 
-bool takes_order(const MarchArgs &a) { return a.n_groups <= 1 && a.near_units == 0; }
+bool takes_order(const MarchArgs &a)
+{
+    if (a.n_groups > 0 || a.n_views == 1) return a.n_groups <= 1;
+    return a.rows_from_middle && static_cast<long long>(a.n_views) * a.width * a.height >= 1 << 17;
+}
 
 const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk, cudaStream_t stream)
 {
@@ -741,8 +746,6 @@ cudaError_t enqueue_regions(Ctx &ctx, const Volume &vol, const std::vector<ViewD
     a.n_views = n;
     a.width = spec.width;
     a.height = spec.height;
-    a.packet_w = cfg.packet_w;
-    a.packet_h = cfg.packet_h;
     a.region = cfg.region;
     double rays = 0.0;
     for (const ViewDev &V : hv) rays += rays_per_cell(V);
@@ -944,7 +947,7 @@ static bool same_kernels(Ctx &ctx, const Volume &vol, const GraphKey &key, const
 
 // Region schedule: the batch is captured from enqueue_regions.
 static int build_region_graph(Ctx &ctx, const Volume &vol, const GraphKey &key, const gbd_image_spec &spec,
-                              const std::vector<ViewDev> &hv, int slots, GraphEntry &g)
+                              const std::vector<ViewDev> &hv, GraphEntry &g)
 {
     const size_t pix = static_cast<size_t>(spec.width) * spec.height * key.n;
     const RegionPlan plan = region_plan(vol, key.cfg, spec, hv);
@@ -975,8 +978,7 @@ static int build_graph(Ctx &ctx, const Volume &vol, const GraphKey &key, const g
                        const std::vector<ViewDev> &hv, GraphEntry &g)
 {
     int nreg[3];
-    const int slots = region_slots(vol, key.cfg, spec, nreg, key.n);
-    if (slots > 0) return build_region_graph(ctx, vol, key, spec, hv, slots, g);
+    if (region_slots(vol, key.cfg, spec, nreg, key.n) > 0) return build_region_graph(ctx, vol, key, spec, hv, g);
     const int n = key.n;
     const size_t pix = static_cast<size_t>(spec.width) * spec.height * n;
     cudaError_t e = cudaSuccess;
@@ -1024,6 +1026,7 @@ int render_graph(Ctx &ctx, const Volume &vol, gbd_volume vid, const std::vector<
     key.samples = spec.out_on_host ? nullptr : spec.samples;
     key.out_on_host = spec.out_on_host;
     key.cfg = cfg;
+    key.cfg.persistent = 0;  // without effect: one graph for both
     GraphCache &gc = *ctx.graphs;
     if (gc.entries.find(key) == gc.entries.end() && gc.entries.size() >= kMaxGraphs) {
         auto oldest = std::min_element(gc.last_use.begin(), gc.last_use.end(),
@@ -1157,8 +1160,6 @@ int gbd_create(gbd_ctx **out, int32_t device, uint64_t hbm_budget_bytes)
     DeviceGuard guard(device);
     auto ctx = std::make_unique<gbd_ctx>();
     ctx->device = device;
-    e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
-    if (e != cudaSuccess) return cuda_fail(e, "multiprocessor count");
     size_t free_b = 0, total_b = 0;
     e = cudaMemGetInfo(&free_b, &total_b);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemGetInfo");
@@ -1525,7 +1526,7 @@ int gbd_render_vector(gbd_ctx *ctx, gbd_volume vid, const gbd_view *views, int32
         a->chan = vol->chan;
         a->chan_comp_stride = vol->chan_stride * vol->grid.n_epochs;
         a->chan_cell_stride = vol->chan_stride;
-        a->block_order = block_order(*ctx, spec->width, spec->height, a->pk, st);
+        if (takes_order(*a)) a->block_order = block_order(*ctx, spec->width, spec->height, a->pk, st);
         e = launch_vector(*a, vol->n_chan, cfg, st);
         ++launches;
     }

@@ -137,7 +137,7 @@ inline PacketGrid packet_grid(int width, int height, int packet_w, int packet_h,
     PacketGrid g;
     g.packet_w = packet_w;
     g.packet_h = packet_h;
-    g.block_w = 1;  // widened while the block stays no wider than high
+    g.block_w = 1;  // widened while the block stays at most twice as wide as high
     while (2 * g.block_w <= cta_warps && 2 * g.block_w * packet_w <= (cta_warps / (2 * g.block_w)) * packet_h * 2) g.block_w *= 2;
     g.step_x = g.block_w * packet_w;
     g.step_y = (cta_warps / g.block_w) * packet_h;
@@ -152,7 +152,8 @@ struct MarchArgs {
     int n_views;              // views in this launch, 1 .. kViewsPerLaunch
     int width, height;
     PacketGrid pk;            // how the CTAs and warps cover an image
-    const int *block_order;   // n-th block that a launch takes of an image (centre first), or NULL: in row order
+    const int *block_order;   // n-th block that a launch takes of an image (centre first), or NULL
+    int rows_from_middle;     // without it: rows of blocks from the middle of the image outwards, or in order
     int n_groups;             // 0: every view marched on its own; else time groups of consecutive views
     int group_size;           // time groups: the kernel's member limit (4 or kGroupMax)
     int group_snaps;          // and its snapshots per cell (kGroupSnapsMin or kGroupSnapsMax)
@@ -203,7 +204,6 @@ struct RegionArgs {
     VolDev vol;
     int n_views;              // views of the batch
     int width, height;
-    int packet_w, packet_h;
     int region;               // region edge in cells
     float rays_per_cell;      // mean of the views (host only: which kernel)
     int nreg[3];              // regions per axis

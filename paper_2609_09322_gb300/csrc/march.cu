@@ -78,7 +78,6 @@ struct BoostConsts {
     float slx, sly, slz;  // rounding residual of s_hat
     float expo;           // 2 - alpha
     bool beaming;
-    bool plain;           // bfloat16/float16 records: D = 1 / (Gamma + u.s_hat) (volume's Gamma <= 8)
 };
 
 template <int STORE>
@@ -103,10 +102,6 @@ struct Record<GBD_STORE_F32> {
         const float inv_g2 = fmaf(-r.y, r.y, fmaf(-r.z, r.z, fmaf(-r.w, r.w, 1.0f)));
         const float log2_d = fmaf(0.5f, lg2_approx(inv_g2), -lg2_approx(den));
         return ex2_approx(c.expo * log2_d);
-    }
-    static __device__ __forceinline__ float boosted(const T r, const BoostConsts &c)
-    {
-        return emissivity(r) * boost(r, c);
     }
 };
 
@@ -146,10 +141,6 @@ struct Record<GBD_STORE_BF16_F16U> {
         const float perp = 1.0f + fmaf(-us, us, uu);
         const float log2_d = (us < 0.f) ? (lg2_approx(gp) - lg2_approx(perp)) : -lg2_approx(gp);
         return ex2_approx(c.expo * log2_d);
-    }
-    static __device__ __forceinline__ float boosted(const T r, const BoostConsts &c)
-    {
-        return emissivity(r) * boost(r, c);
     }
     // boosted2() in the plain form D = 1 / (Gamma + u.s_hat), log2 D =
     // -log2(Gamma + u.s_hat).  For u.s_hat near -Gamma the sum cancels: its
@@ -572,8 +563,8 @@ __device__ __forceinline__ float march_end(const RayState &R, float kk)
 // Byte address of the unit of UNIT bytes (a record, or a pair of them) at layout
 // offset `sum` of block `blk`, blocks blk_bytes apart.  The block term is one 64-bit
 // product of bytes: the same address as (blk * units + sum) << log2(UNIT), in
-// units of a shifted stride, was miscompiled in some kernels (CUDA 13.0: the
-// shift applied to the stride and again to the product).
+// units of a shifted stride, came out with the stride shifted twice in some kernels (CUDA
+// 13.0; their images matched that address and no other).
 template <unsigned UNIT>
 __device__ __forceinline__ unsigned long long rec_addr(unsigned long long base, int blk, long long blk_bytes,
                                                        uint32_t sum)
@@ -669,7 +660,6 @@ __device__ __forceinline__ void march_ray_bf16(const VolDev &vol, const ViewDev 
     bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
     bc.expo = V.expo;
     bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-    bc.plain = PLAIN;
 
     // Block b of the record array (paired: of record pairs) starts b es_bytes
     // from the base.  A sample's lower snapshot m_bar is bp - 1: unpaired, it
@@ -798,7 +788,6 @@ __device__ __forceinline__ void march_ray_exact(const VolDev &vol, const ViewDev
     bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
     bc.expo = V.expo;
     bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-    bc.plain = false;
     // blocks and records as in march_ray_bf16.  Paired float32: a sample that
     // reads no snapshot loads the zero record pair after the last block
     // (faster for 32-byte pairs than a predicated load).
@@ -1004,7 +993,6 @@ __device__ __forceinline__ void march_group(const VolDev &vol, const ViewDev &V,
     bc.slx = V.sh_lo[0]; bc.sly = V.sh_lo[1]; bc.slz = V.sh_lo[2];
     bc.expo = V.expo;
     bc.beaming = (V.flags & GBD_BEAMING) != 0u;
-    bc.plain = PLAIN;
 
     // Unpaired, snapshot m is a record of block m.  Paired, block m holds the
     // records of m - 1 and m side by side: of the snapshots m_0 - k, the even k
@@ -1169,17 +1157,15 @@ __device__ __forceinline__ void block_pixel(const PacketGrid &g, int blocks_x, i
 }
 
 // The march kernels' work split: one CTA per block of packets of one view (or
-// time group), one packet per warp, and the CTAs of the launch view after view.  The
-// hardware hands out CTAs as they end, which balances the load by itself; at any
-// moment the chip works on neighbouring blocks of one or two views, whose rays
-// share cells in L1 (within a CTA) and L2 (against persistent CTAs spread over all views
-// and pulling packets from per-view counters: 24 views of 384^2 of 256^3 x 16 float32 3.17 -> 2.81
-// ms, one 1024^2 image of 512^3 x 8 1.58 -> 1.44 ms).  The view index comes
+// time group), one packet per warp, and the CTAs of the launch run after run (set_runs).  The
+// hardware hands out CTAs as they end, which balances the load by itself, and the
+// rays of a CTA share cells in L1 (against persistent CTAs pulling packets from
+// per-view counters: 24 views of 384^2 of 256^3 x 16 float32 3.09 -> 2.53
+// ms, one 1024^2 image of 512^3 x 8 1.60 -> 1.47 ms).  The view index comes
 // from the CTA index alone, so every per-view constant stays uniform.
 // RUNS: the units of a run (set_runs) go side by side, block by block, instead of one
-// after the other.  bfloat16/float16 groups and vector renders go without: 18 images of 512^2 of a
-// 256^3 x 16 series in bfloat16/float16 groups 431 us without, 477 with; six vector
-// views 864 and 878.
+// after the other.  bfloat16/float16 groups go without: 18 images of 512^2 of a
+// 256^3 x 16 series 431 us, with 477.
 struct BlockWork {
     int unit;   // view, or time group
     int block;  // of its image
@@ -1198,7 +1184,14 @@ __device__ __forceinline__ BlockWork block_work(const MarchArgs &a)
     } else {
         w.block = b - w.unit * a.pk.blocks;
     }
-    if (a.block_order) w.block = __ldg(a.block_order + w.block);
+    if (a.block_order) {
+        w.block = __ldg(a.block_order + w.block);
+    } else if (RUNS && a.rows_from_middle) {
+        // rows of blocks m, m - 1, m + 1, m - 2, ... from the middle one, m
+        const int row = w.block / a.pk.blocks_x, half = (row + 1) >> 1;
+        const int to = ((a.pk.blocks / a.pk.blocks_x) >> 1) + ((row & 1) ? -half : half);
+        w.block += (to - row) * a.pk.blocks_x;
+    }
     return w;
 }
 
@@ -1256,12 +1249,16 @@ __global__ void __launch_bounds__(256, 3) group_kernel(const __grid_constant__ M
 // Vector renders: march_kernel's work split with NCH extra channels summed
 // along every ray (stages of one cell, at most 96 registers: six views of 384^2 of
 // 192^3 x 8 with three channels 878 us at the compiler's 106, 854 at 96, 897 at 80).
-template <int STORE, int NCH, bool PAIRED>
+// RUNS: side by side (set_runs) for launches of kRunsPixels and more; below, the run's arithmetic
+// costs each ray's latency more than the order gains (three channels of 3 views of 64^2 of 160^3
+// 182 us without, 191 with; of 4 of 192^2 327 and 271).
+constexpr long long kRunsPixels = 1 << 17;
+template <int STORE, int NCH, bool PAIRED, bool RUNS>
 __global__ void __maxnreg__(96) vector_kernel(const __grid_constant__ MarchArgs a)
 {
     extern __shared__ int32_t s_mem[];
     int32_t *s_tab = s_mem + kSpanEntries;
-    const BlockWork w = block_work<true>(a);
+    const BlockWork w = block_work<RUNS>(a);
     const ViewDev &V = a.views[w.unit];
     int p, q;
     block_pixel(a.pk, a.pk.blocks_x, w.block, p, q);
@@ -1334,10 +1331,8 @@ __global__ void __launch_bounds__(256, MINB) wave_kernel(const __grid_constant__
 // region y.  The region's table entries along each axis (forward or reversed,
 // as the view needs) are staged in shared memory.
 // The view's pixels whose rays can cross the region lie in the projection of
-// the region's box; the CTA takes one packet of that rectangle per warp,
-// keeps the rays that cross the box, sorts them by the length of their chord
-// through it (8 buckets, longest first) and hands them to its warps 32 at a
-// time, so that the rays of a warp end at about the same step.  Each ray adds
+// the region's box; screen_kernel lists them, longest chord first, and each warp takes
+// the next 32 of the list, so that its rays end at about the same step.  Each ray adds
 // its region sum to its partial slot.
 // Region r of view vi: its box in the view's march frame (mirrored axes
 // mirrored) with the offsets of its staged march tables, its partial slot, and
@@ -1733,16 +1728,24 @@ void *select_region(int store, int depth, int capped, int paired, bool sparse)
     return nullptr;
 }
 
-template <int NCH>
+template <int NCH, bool RUNS>
 void *select_vector_store(int store, int paired)
 {
     if (store == GBD_STORE_F32)
-        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, true>)
-                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, false>);
+        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, true, RUNS>)
+                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_F32, NCH, false, RUNS>);
     if (store == GBD_STORE_BF16_F16U)
-        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, true>)
-                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, false>);
+        return paired ? reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, true, RUNS>)
+                      : reinterpret_cast<void *>(&vector_kernel<GBD_STORE_BF16_F16U, NCH, false, RUNS>);
     return nullptr;
+}
+
+template <int NCH>
+void *select_vector_runs(const MarchArgs &a)
+{
+    const bool runs = a.n_views > 1 && static_cast<long long>(a.n_views) * a.width * a.height >= kRunsPixels;
+    return runs ? select_vector_store<NCH, true>(a.vol.store, a.vol.paired)
+                : select_vector_store<NCH, false>(a.vol.store, a.vol.paired);
 }
 
 void *select_wave(int depth, int capped)
@@ -1774,8 +1777,7 @@ cudaError_t launch_wave(const WaveArgs &a, const LaunchCfg &cfg, cudaStream_t st
 
 cudaError_t launch_vector(MarchArgs &a, int n_chan, const LaunchCfg &cfg, cudaStream_t stream)
 {
-    void *k = n_chan == 1 ? select_vector_store<1>(a.vol.store, a.vol.paired)
-                          : (n_chan == 3 ? select_vector_store<3>(a.vol.store, a.vol.paired) : nullptr);
+    void *k = n_chan == 1 ? select_vector_runs<1>(a) : (n_chan == 3 ? select_vector_runs<3>(a) : nullptr);
     if (!k) return cudaErrorInvalidValue;
     // grid and shared memory as planned for the scalar kernel
     KernelLaunch L;

@@ -21,7 +21,7 @@ namespace {
 constexpr int kNoAllocMaxViews = GBD_NOALLOC_MAX_VIEWS;
 std::mutex g_mu;                          // guards the arrays below
 ViewDev g_host_views[kNoAllocMaxViews];   // the views, set up on the host
-MarchArgs g_args;                         // launch arguments (about 28 KB: not on the stack)
+MarchArgs g_args;                         // launch arguments (about 31 KB: not on the stack)
 
 }  // namespace
 }  // namespace gbd

@@ -59,7 +59,6 @@ struct TuneEntry {
 
 struct gbd_ctx {
     int device = 0;
-    int num_sms = 0;
     uint64_t budget = 0;
     uint64_t used = 0;
     std::mutex mu;
@@ -141,11 +140,16 @@ void group_views(MarchArgs &a, int gmax);
 // The order in which a launch takes an image's blocks: by distance of the block from the
 // image centre, nearest first (the longest rays of a centred box first, so the launch
 // ends on short ones).  A device table cached in the context for up to 64 image
-// geometries; NULL (row order) beyond them, if it cannot be made, or on its first use while `stream` is captured.
+// geometries; NULL beyond them, if it cannot be made, or on its first use while
+// `stream` is captured.
 const int *block_order(Ctx &ctx, int width, int height, const PacketGrid &pk, cudaStream_t stream);
-// The launches that use it: all but those of several time groups or of views within a
-// snapshot of each other along the same rays, whose neighbouring CTAs share more on
-// neighbouring blocks (24 views 0.1 snapshots apart, paired float32: 1025 us, in this order 1073).
+// The launches that use it: of one view or time group, and of views along different rays
+// with 2^17 pixels and more.  Smaller ones of those take the rows of blocks from the
+// middle outwards, which needs no table (25 us on the first use, 1 us a launch; 8
+// views of 128^2, 2^17 pixels, of three channels of 160^3 x 6 305 us by table, 320 by rows).  Several time
+// groups, and views within a snapshot of each other along the same rays, keep
+// neighbouring CTAs on neighbouring blocks (24 views 0.1 snapshots apart, paired float32:
+// 1025 us, by table 1073).
 bool takes_order(const MarchArgs &a);
 bool build_layout(const int n[3], int B, int S, std::vector<int32_t> &tab, long long &epoch_stride, int morton_cells);
 void destroy_graph_cache(GraphCache *g);
