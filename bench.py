@@ -64,8 +64,9 @@ RECORD_BYTES = {"f32": 16, "bf16": 8}
 
 # Launch (packet_w, packet_h, warps per CTA, cells ahead, capped registers
 # [, region edge [, time-group size]]) and layout (brick, super-brick, paired)
-# measured fastest on GB300 for each workload, within the autotuner's search
-# space.
+# measured fastest on GB300 for each workload and form, within the autotuner's
+# search space ("time_delay" is the form that marches each view on its own; time groups,
+# "time_delay_grouped", are faster).
 PINNED = {
     "batched": ("4,8,4,2,1,64", "8,4,0"),
     "batched_bf16": ("4,8,4,2,1,64", "4,4,1"),

@@ -466,8 +466,7 @@ class Context:
 
     def render_batch_noalloc(self, vol: int, views, out, *, launch=None, stream=None):
         """``render_batch`` into the caller's device tensor ``out`` [n][H][W]
-        without any allocation by the library (its scratch is a fixed
-        device array; at most 1024 views per call).  ``out`` must be a
+        without any allocation by the library (at most 1024 views per call).  ``out`` must be a
         contiguous float32 tensor of shape [n][H][W] on this context's device:
         the library writes n * H * W floats from its first element."""
         import torch
